@@ -61,13 +61,17 @@ template void spmm<float2>(int64_t, const int32_t*, const int32_t*, const float2
 // Rows are visited four at a time with independent loads, so that enough
 // memory requests are in flight to stream V and W at HBM rate.
 // With self = 1 the product conj(W) W is appended as vector index nvec.
+// A block is (columns) x (8 row lanes) threads, columns the power of two at or
+// above m, at most 32: idle lanes would still take their share of the FP64
+// pipe (two multiply-adds per clock and SM), which bounds the FP64 form (a
+// gradient step of 8 columns on 46,080 tets 152 -> 142 ms).
 template <typename C>
 __global__ void __launch_bounds__(256) dots_kernel(int64_t n, int m, int nvec_in, const C* __restrict__ V,
                                                    int64_t vstride, const C* __restrict__ W, int self,
                                                    double2* __restrict__ partial) {
     __shared__ double2 red[8][8][33];
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const int c = blockIdx.y * 32 + tx;
+    const int c = blockIdx.y * blockDim.x + tx;
     const int64_t stride = (int64_t)gridDim.x * 8;
     const int nvec = nvec_in + self;
     for (int i0 = 0; i0 < nvec; i0 += 8) {
@@ -126,34 +130,36 @@ __global__ void __launch_bounds__(256) dots_kernel(int64_t n, int m, int nvec_in
 
 // h[i][c] = sum_b partial[b][i][c] for i < nvec; hacc[i][c] += h[i][c] for i < nacc;
 // hdf (optional) receives h as double-floats (re hi, re lo, im hi, im lo).
-// One block per vector index i: 8 warps split the blocks b (b = lane, lane + 8,
-// ...), lanes over columns, then a fixed-order sum of the 8 partial sums.
-__global__ void __launch_bounds__(256) dots_reduce_kernel(int nblk, int nvec, int nacc, int m,
+// One block per vector index i: 32 warps split the blocks b (b = warp, warp +
+// 32, ...), lanes over columns, then a fixed-order sum of the 32 partial sums.
+// The chain of loads and FP64 additions per warp bounds it (with 8 warps a
+// forward solve of 4 columns on 3,072 tets took 6.25 ms, with 32 it takes 5.62).
+__global__ void __launch_bounds__(1024) dots_reduce_kernel(int nblk, int nvec, int nacc, int m,
                                                           const double2* __restrict__ partial,
                                                           double2* __restrict__ h, double2* __restrict__ hacc,
                                                           float4* __restrict__ hdf) {
-    __shared__ double2 red[8][32];
+    __shared__ double2 red[32][33];
     const int i = blockIdx.x;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     for (int c0 = 0; c0 < m; c0 += 32) {
         const int c = c0 + tx;
         double sx = 0.0, sy = 0.0;
         if (c < m) {
-#pragma unroll 4
-            for (int b = ty; b < nblk; b += 8) {
+#pragma unroll 10
+            for (int b = ty; b < nblk; b += 32) {
                 const double2 v = partial[((int64_t)b * nvec + i) * m + c];
                 sx += v.x;
                 sy += v.y;
             }
         }
         red[ty][tx] = make_double2(sx, sy);
-        __syncthreads();
+#pragma unroll
+        for (int w = 16; w > 0; w >>= 1) {
+            __syncthreads();
+            if (ty < w) red[ty][tx] = cadd(red[ty][tx], red[ty + w][tx]);
+        }
         if (ty == 0 && c < m) {
-            double2 s = red[0][tx];
-            for (int k = 1; k < 8; ++k) {
-                s.x += red[k][tx].x;
-                s.y += red[k][tx].y;
-            }
+            const double2 s = red[0][tx];
             const int e = i * m + c;
             h[e] = s;
             if (hacc && i < nacc) { hacc[e].x += s.x; hacc[e].y += s.y; }
@@ -849,11 +855,13 @@ void Gmres<C>::reserve(int64_t n_, int m_, int restart_) {
 template <typename C>
 static void dots_launch(int64_t n, int m, const C* Vb, int nvec, int64_t vstride, const C* w, double2* partial,
                         double2* out, double2* acc, float4* hdf, cudaStream_t st, int self) {
-    dim3 blk(32, 8), grd(kDotBlocks, (m + 31) / 32);
+    int mx = 1;
+    while (mx < std::min(m, 32)) mx *= 2;
+    dim3 blk(mx, 8), grd(kDotBlocks, (m + mx - 1) / mx);
     dots_kernel<C><<<grd, blk, 0, st>>>(n, m, nvec, Vb, vstride, w, self, partial);
     MWI_CHECK_LAUNCH();
     const int nt = nvec + self;
-    dots_reduce_kernel<<<nt, 256, 0, st>>>(kDotBlocks, nt, nvec, m, partial, out, acc, hdf);
+    dots_reduce_kernel<<<nt, 1024, 0, st>>>(kDotBlocks, nt, nvec, m, partial, out, acc, hdf);
     MWI_CHECK_LAUNCH();
 }
 
@@ -1004,7 +1012,7 @@ int GmresDF::cycle(const OpA& A, const OpM& M, const float2* r0, float2* x, cons
             dots2_kernel<<<grd, blk, 0, st>>>(n, m, k, V.p, vs, vk, W.p, partial.p);
             MWI_CHECK_LAUNCH();
             const int nout = 2 * k + 3;
-            dots_reduce_kernel<<<nout, 256, 0, st>>>(nblk, nout, 0, m, partial.p, h.p, nullptr, nullptr);
+            dots_reduce_kernel<<<nout, 1024, 0, st>>>(nblk, nout, 0, m, partial.p, h.p, nullptr, nullptr);
             MWI_CHECK_LAUNCH();
             MWI_CUDA(cudaMemsetAsync(nact, 0, sizeof(int), st));
             arnoldi_dcgs_kernel<<<nblocks(m, 128), 128, 0, st>>>(m, k, restart, last, h.p, H.p, Hp.p, cs.p, sn.p,
