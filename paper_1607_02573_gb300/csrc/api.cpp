@@ -148,6 +148,7 @@ struct mwi_problem {
     DevBuf<float2> ws32, inv32, sch32[2];
     DevBuf<float> wt;        // tiled, swizzled copy of the c64 panels (tensor-core sweeps)
     DevBuf<int> sweep_err;   // error code of the tensor-core sweeps' bounded waits
+    DevBuf<int> sweep_cnt;   // their completion counts (one application at a time: the problem's stream)
     DevBuf<int> perturbed;
     int n_perturbed = 0;
     // solve state
@@ -210,7 +211,7 @@ struct mwi_problem {
                    rx_dof_d.bytes() + tx_dof_d.bytes() + rx_sign_d.bytes() + tx_sign_d.bytes() + cur_d.bytes() +
                    S_d.bytes() + Smeas_d.bytes() + r_d.bytes() + grad_d.bytes() + w_d.bytes() + J_d.bytes() +
                    kappa.bytes() + Mk.bytes() + grad_tw.bytes() + p1_partial.bytes() + nonfinite.bytes() +
-                   wt.bytes() + sweep_err.bytes();
+                   wt.bytes() + sweep_err.bytes() + sweep_cnt.bytes();
         for (int k = 0; k < 2; ++k) b += sch64[k].bytes() + sch32[k].bytes();
         if (coarse) b += coarse->bytes();
         return b;
@@ -265,6 +266,7 @@ SweepCfg sweep_cfg(const mwi_problem* P) {
     c.tc = tc_of(P->opts);
     c.wt = P->wt.p;
     c.err = P->sweep_err.p;
+    c.cnt = P->sweep_cnt.p;
     return c;
 }
 
@@ -408,7 +410,13 @@ void upload_fronts(const Decomposition& D, FrontsDev& F, cudaStream_t st) {
     up(F.start, start, st); up(F.p, p, st); up(F.u, u, st); up(F.parent, parent, st); up(F.sub, sub, st);
     up(F.f_off, f_off, st); up(F.u_off, u_off, st); up(F.upd_row, upd_row, st); up(F.sch_off, sch_off, st);
     up(F.child_ptr, D.child_ptr, st); up(F.child, D.child, st);
-    up(F.urows, D.urows, st); up(F.urel, D.urel, st);
+    {
+        // padded: the sweeps copy index lists in 16-byte units
+        std::vector<int32_t> ur(D.urows);
+        ur.resize(ur.size() + 8, 0);
+        up(F.urows, ur, st);
+    }
+    up(F.urel, D.urel, st);
     up(F.asm_base, D.asm_base, st); up(F.asm_ptr, D.asm_ptr, st); up(F.asm_src, D.asm_src, st);
     {
         // every front row receives at most one row from each of its (at most two) children
@@ -534,42 +542,86 @@ void upload_fronts(const Decomposition& D, FrontsDev& F, cudaStream_t st) {
         if (pb.empty()) pb.push_back(make_int2(0, 0));
         up(F.t_off, toff, st);
         up(F.pack_blocks, pb, st);
-        TileLists& TL = F.tiles128;
-        TL.tm = 128;
-        std::vector<TileDesc> pt, ft;
-        TL.p_ptr.assign(1, 0);
-        TL.f_ptr.assign(1, 0);
-        for (int l = 0; l < nlev; ++l) {
-            for (int q = D.level_ptr[l]; q < D.level_ptr[l + 1]; ++q) {
-                const int sid = D.level_fronts[q];
-                const Front& fr = D.fronts[sid];
-                TileDesc d;
-                d.a_off = toff[sid];
-                d.sbase = D.sub_off[fr.sub];
-                d.rowbase = d.sbase + fr.start;
-                d.upd_row = fr.upd_row;
-                d.asm_base = D.asm_base[sid];
-                d.u_off = fr.u_off;
-                d.p = fr.p;
-                d.f = fr.p + fr.u;
-                d.pad = 0;
-                for (int r = 0; r < fr.p; r += 128) { d.row0 = r; pt.push_back(d); }
-                for (int r = 0; r < fr.p + fr.u; r += 128) { d.row0 = r; ft.push_back(d); }
+        // sweep tiles in the order they are drawn; a front's counts: forward 1 + s,
+        // backward 1 + nf + s, four (one per epilogue warp) for every tile and chunk
+        auto tiles_of = [&](size_t s, bool bwd) {
+            const Front& fr = D.fronts[s];
+            return ((bwd ? fr.p : fr.p + fr.u) + 127) / 128;
+        };
+        std::vector<TcTile> tl;
+        auto push = [&](int sid, bool bwd) {
+            const Front& fr = D.fronts[sid];
+            TcTile d{};
+            d.a_off = toff[sid] + (bwd ? F.tiled_floats : 0);
+            d.sbase = D.sub_off[fr.sub];
+            d.rowbase = d.sbase + fr.start;
+            d.upd_row = fr.upd_row;
+            d.asm_base = D.asm_base[sid];
+            d.u_off = fr.u_off;
+            d.p = fr.p;
+            d.f = fr.p + fr.u;
+            d.bwd = bwd ? 1 : 0;
+            d.cnt = (int32_t)(1 + (bwd ? nf : 0) + sid);
+            d.dep0 = d.dep1 = d.sib = -1;
+            if (bwd) {
+                const bool root = fr.parent < 0;
+                d.dep0 = (int32_t)(root ? 1 + sid : 1 + nf + fr.parent);
+                d.need0 = 4 * (root ? tiles_of(sid, false) : tiles_of(fr.parent, true));
+            } else {
+                const int c0 = D.child_ptr[sid], c1 = D.child_ptr[sid + 1];
+                if (c1 > c0) {
+                    d.dep0 = 1 + D.child[c0];
+                    d.need0 = 4 * tiles_of(D.child[c0], false);
+                }
+                if (c1 > c0 + 1) {
+                    d.dep1 = 1 + D.child[c0 + 1];
+                    d.need1 = 4 * tiles_of(D.child[c0 + 1], false);
+                }
+                if (fr.parent >= 0) {
+                    const int first = D.child[D.child_ptr[fr.parent]];
+                    if (first != sid) {
+                        d.sib = 1 + first;
+                        d.needs = 4 * tiles_of(first, false);
+                    }
+                }
             }
-            // heaviest first (stages per tile): backward by row blocks, forward by pivot atoms
-            std::stable_sort(pt.begin() + TL.p_ptr.back(), pt.end(), [](const TileDesc& a, const TileDesc& b) {
-                return (a.f + 31) / 32 - a.row0 / 32 > (b.f + 31) / 32 - b.row0 / 32;
-            });
-            std::stable_sort(ft.begin() + TL.f_ptr.back(), ft.end(), [](const TileDesc& a, const TileDesc& b) {
-                return std::min(a.p, a.row0 + 128) > std::min(b.p, b.row0 + 128);
-            });
-            TL.p_ptr.push_back((int64_t)pt.size());
-            TL.f_ptr.push_back((int64_t)ft.size());
+            // heaviest tile of the front first
+            const int t = tiles_of(sid, bwd);
+            for (int k = 0; k < t; ++k) {
+                d.row0 = 128 * (bwd ? k : t - 1 - k);
+                tl.push_back(d);
+            }
+        };
+        F.tc_level_fwd.assign(nlev, 0);
+        F.tc_level_bwd.assign(nlev, 0);
+        for (int pass = 0; pass < 2; ++pass)
+            for (int k = 0; k < nlev; ++k) {
+                const int l = pass ? nlev - 1 - k : k;
+                const size_t before = tl.size();
+                // forward: the first children before the second ones, which add to the
+                // parent's rows after them
+                for (int second = 0; second < (pass ? 1 : 2); ++second)
+                    for (int q = D.level_ptr[l]; q < D.level_ptr[l + 1]; ++q) {
+                        const int sid = D.level_fronts[q], par = D.fronts[sid].parent;
+                        const bool is2 = !pass && par >= 0 && D.child[D.child_ptr[par]] != sid;
+                        if (is2 == (second != 0)) push(sid, pass != 0);
+                    }
+                (pass ? F.tc_level_bwd : F.tc_level_fwd)[l] = (int64_t)(tl.size() - before);
+            }
+        F.tc_ntiles = (int64_t)tl.size();
+        if (tl.empty()) tl.push_back(TcTile{});
+        F.tc_tiles.upload(tl, st);
+        std::vector<int32_t> pd(std::max<int64_t>(1, D.upd_rows), -1);
+        for (size_t c = 0; c < nf; ++c) {
+            const Front& fr = D.fronts[c];
+            if (fr.parent < 0) continue;
+            const Front& pa = D.fronts[fr.parent];
+            for (int j = 0; j < fr.u; ++j) {
+                const int32_t rel = D.urel[fr.u_off + j];
+                if (rel < pa.p) pd[fr.upd_row + j] = (int32_t)(D.sub_off[pa.sub] + pa.start + rel);
+            }
         }
-        if (pt.empty()) pt.push_back(TileDesc{});
-        if (ft.empty()) ft.push_back(TileDesc{});
-        TL.p_tiles.upload(pt, st);
-        TL.f_tiles.upload(ft, st);
+        up(F.pdst, pd, st);
     }
     {
         std::vector<int64_t> io(D.level_fronts.size());
@@ -767,6 +819,7 @@ void numeric_setup(mwi_problem* P, bool refactor = true) {
             }
         });
         if (tc_of(P->opts) == 4 && !P->sweep_err.p) {
+            P->sweep_cnt.alloc(E.F.tc_counts());
             P->sweep_err.alloc(1);
             MWI_CUDA(cudaMemsetAsync(P->sweep_err.p, 0, sizeof(int), st));
         }
@@ -1758,8 +1811,8 @@ mwi_status mwi_sweep_levels(mwi_problem_t P, int32_t max_levels, int32_t* n_leve
             if (fronts) fronts[l] = D.level_ptr[l + 1] - D.level_ptr[l];
             if (panel_entries) panel_entries[l] = e;
             if (update_rows) update_rows[l] = u;
-            if (tiles_fwd) tiles_fwd[l] = F.tiles128.f_ptr[l + 1] - F.tiles128.f_ptr[l];
-            if (tiles_bwd) tiles_bwd[l] = F.tiles128.p_ptr[l + 1] - F.tiles128.p_ptr[l];
+            if (tiles_fwd) tiles_fwd[l] = F.tc_level_fwd[l];
+            if (tiles_bwd) tiles_bwd[l] = F.tc_level_bwd[l];
         }
     });
 }
@@ -1812,7 +1865,7 @@ mwi_status mwi_problem_estimate_bytes(mwi_mesh_t M, const mwi_solver_opts* opts,
                    (double)E->B.nnz * 16;
         b += nested ? nnz * 8 : (mixed ? 2 * nnz * 8 : 0);
         b += ((double)F.ws_total() + (double)F.inv_entries + (double)F.sch_entries[0] + (double)F.sch_entries[1]) * fe;
-        if (mixed && o.sweep_engine == 4) b += 2.0 * (double)F.tiled_floats * 4;
+        if (mixed && o.sweep_engine == 4) b += 2.0 * (double)F.tiled_floats * 4 + 4.0 * (double)F.tc_counts();
         // fields of every column (forward, adjoint, right-hand sides), block copies, residual
         b += 3 * n * mall * 16 + 3 * n * m * 16;
         // local and update vectors of the ORAS application

@@ -83,13 +83,31 @@ struct TileLists {
     std::vector<int64_t> p_ptr, f_ptr;  // [n_levels+1]
 };
 
+// One 128-row tile of the tensor-core sweeps (sweep_tc.cu): the front's
+// geometry (a_off: its panel copy of the tile's direction, in floats), the
+// front's completion count that the tile adds to, the counts it waits for
+// (-1: none) and their values per column chunk; sib: of the first child, for
+// the tiles of a second one.  Counts are indices into one int array whose
+// entry 0 draws the tiles.
+struct __align__(8) TcTile {
+    int64_t a_off, rowbase, sbase, upd_row, asm_base, u_off;
+    int32_t p, f, row0, bwd;
+    int32_t cnt, dep0, need0, dep1, need1, sib, needs, pad;
+};
+
 struct FrontsDev {
     int64_t nfronts = 0;
-    // tensor-core sweeps (sweep_tc.cu): 128-row tiles whose a_off is the
-    // front's offset in each tiled copy of the panels (floats), the per-front
-    // offsets, the (front, 32-row block) list of the packing kernel, and the
-    // floats of one copy (the store holds the forward then the backward copy)
-    TileLists tiles128;
+    // tensor-core sweeps: the tiles in the order they are drawn, tile counts per
+    // level (forward, backward), per update row the parent's pivot row in the
+    // local vectors that it adds to (-1: an update row of the parent), the
+    // per-front offsets in each tiled copy of the panels, the (front, 32-row
+    // block) list of the packing kernel, and the floats of one copy (the store
+    // holds the forward then the backward copy)
+    DevBuf<TcTile> tc_tiles;
+    int64_t tc_ntiles = 0;
+    std::vector<int64_t> tc_level_fwd, tc_level_bwd;
+    DevBuf<int32_t> pdst;
+    int64_t tc_counts() const { return 1 + 2 * nfronts; }
     DevBuf<int64_t> t_off;
     DevBuf<int2> pack_blocks;
     int64_t n_pack_blocks = 0, tiled_floats = 0;
@@ -148,11 +166,13 @@ void factorize_fronts(const FrontsDev& F, const UpdateTiles& ut, const double2* 
                       C* inv_tmp, int* perturbed, cudaStream_t st);
 
 // Complex FP32 sweep engine: tc = 0 CUDA cores, 1 mma.sync 3xTF32, 2 mma.sync
-// TF32, 4 tcgen05 TF32 over the tiled panel store wt (err: the kernels'
+// TF32, 4 tcgen05 TF32 over the tiled panel store wt (cnt: FrontsDev::tc_counts()
+// ints of the caller's, used by one application at a time; err: the kernels'
 // bounded-wait error code, 0 = none)
 struct SweepCfg {
     int tc = 0;
     const float* wt = nullptr;
+    int* cnt = nullptr;
     int* err = nullptr;
 };
 
@@ -173,9 +193,8 @@ int64_t tiled_panel_floats(int p, int f);
 // both tiled copies: the forward one at wt, the backward one at wt + bwd_base
 void pack_tiled(const int2* blocks, int64_t nblocks, const int64_t* f_off, const int64_t* t_off, const int32_t* P,
                 const int32_t* U, const float2* ws, float* wt, int64_t bwd_base, cudaStream_t st);
-void sweep_tc_level(bool backward, const TileDesc* tiles, int64_t ntiles, int m, const int32_t* urows,
-                    const int2* asm2, const float* wt, const float2* dinv, float2* Y, float2* Z, float2* upd,
-                    int* err, cudaStream_t st);
+void sweep_tc_solve(const FrontsDev& F, int m, const float* wt, const float2* dinv, float2* Y, float2* Z,
+                    float2* upd, int* cnt, int* err, cudaStream_t st);
 
 // Allocation-free ORAS application (oras.cu): scratch from a fixed-size
 // file-scope device array of kOrasScratchBytes.

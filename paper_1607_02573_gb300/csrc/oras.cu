@@ -26,11 +26,14 @@ template <> __device__ __forceinline__ float2 cvt<float2, float2>(float2 v) { re
 template <> __device__ __forceinline__ float2 cvt<double2, float2>(double2 v) { return make_float2((float)v.x, (float)v.y); }
 template <> __device__ __forceinline__ double2 cvt<float2, double2>(float2 v) { return make_double2(v.x, v.y); }
 
-// local vectors have ld >= m columns; the columns m..ld-1 are zero
+// local vectors have ld >= m columns; the columns m..ld-1 are zero.  cnt
+// (nullable): the tensor-core sweeps' counts, cleared on the way
 template <typename In, typename C>
 __global__ void gather_kernel(int64_t nloc, int m, int ld, const int32_t* __restrict__ loc2glob,
-                              const In* __restrict__ x, C* __restrict__ Y) {
+                              const In* __restrict__ x, C* __restrict__ Y, int* __restrict__ cnt, int ncnt) {
     int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (cnt)
+        for (int64_t q = e; q < ncnt; q += (int64_t)gridDim.x * blockDim.x) cnt[q] = 0;
     if (e >= nloc * ld) return;
     int64_t r = e / ld;
     int c = (int)(e - r * ld);
@@ -60,8 +63,12 @@ __global__ void scatter_kernel(int64_t n, int m, int ld, const int64_t* __restri
 // columns (16 bytes) per thread: a block of (threads per row) x (rows), so no
 // thread divides by the row length
 __global__ void gather2_kernel(int64_t nloc, int h, int ldh, const int32_t* __restrict__ loc2glob,
-                               const float4* __restrict__ x, float4* __restrict__ Y) {
+                               const float4* __restrict__ x, float4* __restrict__ Y, int* __restrict__ cnt,
+                               int ncnt) {
     const int64_t r = blockIdx.x * (int64_t)blockDim.y + threadIdx.y;
+    if (cnt)
+        for (int64_t q = r * blockDim.x + threadIdx.x; q < ncnt; q += (int64_t)gridDim.x * blockDim.x * blockDim.y)
+            cnt[q] = 0;
     if (r >= nloc) return;
     const int64_t g = loc2glob[r];
     for (int c = threadIdx.x; c < ldh; c += blockDim.x)
@@ -108,13 +115,17 @@ static void oras_apply_impl(const FrontsDev& F, const C* ws, const In* x, Out* y
                          std::is_same<Out, float2>::value;
     const bool pairs = c64 && (m % 2) == 0 && (ld % 2) == 0;
     const int64_t n = (int64_t)F.own_ptr.n - 1;
+    int* cnt = std::is_same<C, float2>::value && sc.tc == 4 ? sc.cnt : nullptr;
+    const int ncnt = (int)F.tc_counts();
     if (pairs) {
         const dim3 b = pair_block(m / 2);
         gather2_kernel<<<(unsigned)((F.nloc + b.y - 1) / b.y), b, 0, st>>>(
-            F.nloc, m / 2, ld / 2, F.loc2glob.p, reinterpret_cast<const float4*>(x), reinterpret_cast<float4*>(Y));
+            F.nloc, m / 2, ld / 2, F.loc2glob.p, reinterpret_cast<const float4*>(x), reinterpret_cast<float4*>(Y), cnt,
+            ncnt);
     } else {
         const int64_t tot = F.nloc * ld;
-        gather_kernel<In, C><<<(unsigned)((tot + th - 1) / th), th, 0, st>>>(F.nloc, m, ld, F.loc2glob.p, x, Y);
+        gather_kernel<In, C><<<(unsigned)((tot + th - 1) / th), th, 0, st>>>(F.nloc, m, ld, F.loc2glob.p, x, Y, cnt,
+                                                                                 ncnt);
     }
     MWI_CHECK_LAUNCH();
     multifrontal_solve<C>(F, ws, Y, Z, upd, ld, sc, st);

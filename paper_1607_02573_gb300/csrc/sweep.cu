@@ -603,44 +603,25 @@ static void launch_gather(const FrontsDev& F, int l, C* Y, const C* upd, int m, 
     MWI_CHECK_LAUNCH();
 }
 
-// one level's product on the fifth-generation tensor cores (sweep_tc.cu)
-template <typename C>
-static void launch_tc_product(const FrontsDev& F, int l, bool backward, const C* ws, C* Y, C* Z, C* upd, int m,
-                              const SweepCfg& sc, cudaStream_t st) {
-    if constexpr (std::is_same<C, float2>::value) {
-        const TileLists& T = F.tiles128;
-        const int64_t b = backward ? T.p_ptr[l] : T.f_ptr[l];
-        const int64_t e = backward ? T.p_ptr[l + 1] : T.f_ptr[l + 1];
-        sweep_tc_level(backward, (backward ? T.p_tiles.p : T.f_tiles.p) + b, e - b, m, F.urows.p, F.asm2.p,
-                       sc.wt + (backward ? F.tiled_floats : 0), ws + F.ws_entries, Y, Z, upd, sc.err, st);
-    } else {
-        throw Error(MWI_EINVAL, "internal: tensor-core sweeps need complex FP32 factors");
-    }
-}
-
 template <typename C>
 void multifrontal_solve(const FrontsDev& F, const C* ws, C* Y, C* Z, C* upd, int m, const SweepCfg& sc,
                         cudaStream_t st) {
+    if constexpr (std::is_same<C, float2>::value) {
+        if (sc.tc == 4) {
+            // the tcgen05 engine moves right-hand-side rows by 16-byte bulk copies
+            // (oras_apply pads the local vectors to an even column count)
+            MWI_REQUIRE(sc.wt && sc.err && sc.cnt, MWI_EINVAL, "internal: tensor-core sweeps without their buffers");
+            MWI_REQUIRE((m % 2) == 0, MWI_EINVAL, "internal: tensor-core sweeps need an even column count");
+            sweep_tc_solve(F, m, sc.wt, ws + F.ws_entries, Y, Z, upd, sc.cnt, sc.err, st);
+            return;
+        }
+    }
     const int nlev = (int)F.level_ptr.size() - 1;
-    // the tcgen05 engine moves right-hand-side rows by 16-byte bulk copies
-    // (oras_apply pads the local vectors to an even column count)
-    const bool tc5 = sc.tc == 4;
-    const int tc = sc.tc;
-    MWI_REQUIRE(!tc5 || (sc.wt && sc.err), MWI_EINVAL, "internal: tensor-core sweeps without the tiled panels");
-    MWI_REQUIRE(!tc5 || (m % 2) == 0, MWI_EINVAL, "internal: tensor-core sweeps need an even column count");
     for (int l = 0; l < nlev; ++l) {
         launch_gather<C>(F, l, Y, upd, m, st);
-        if (tc5) launch_tc_product<C>(F, l, false, ws, Y, Z, upd, m, sc, st);
-        else launch_gemm<C, kFwd>(F, l, ws, Y, Z, upd, m, tc, st);
+        launch_gemm<C, kFwd>(F, l, ws, Y, Z, upd, m, sc.tc, st);
     }
-    // backward levels of small fronts (mean pivot count below 40): the TF32
-    // mma.sync kernel with 32-row tiles beats the 128-row tcgen05 tiles there
-    // (one tile per front either way; the per-tile pipeline set-up of the
-    // tcgen05 kernel dominates), so the tcgen05 engine hands those levels to it
-    for (int l = nlev - 1; l >= 0; --l) {
-        if (tc5 && !small_tiles<C>(F, l, false)) launch_tc_product<C>(F, l, true, ws, Y, Z, upd, m, sc, st);
-        else launch_gemm<C, kBwd>(F, l, ws, Y, Z, upd, m, tc5 ? 2 : tc, st);
-    }
+    for (int l = nlev - 1; l >= 0; --l) launch_gemm<C, kBwd>(F, l, ws, Y, Z, upd, m, sc.tc, st);
 }
 
 template void multifrontal_solve<float2>(const FrontsDev&, const float2*, float2*, float2*, float2*, int,

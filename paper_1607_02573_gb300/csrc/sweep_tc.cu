@@ -19,10 +19,13 @@
 //     tile is 16 consecutive blocks (row groups at the stride-byte offset);
 //   - backward copy: line = pivot, 8 floats = front rows; blocks ordered
 //     [row chunk][pivot group][plane].
-// A stage of 32 K values is at most four contiguous byte ranges, copied with
-// cp.async.bulk.  The right-hand sides are written K-major into the B stage by
-// the gather warps (line = real column, 32 floats = the stage's K rows,
-// 128-byte swizzle).
+// A stage of kKS K steps is at most kKS contiguous byte ranges, copied with
+// cp.async.bulk.  The right-hand sides are the B operand as they lie in memory,
+// N contiguous (MN-major): the TF32 form takes that in one layout only, the
+// 128-byte swizzle of 32-byte atoms -- 128 bytes (32 real columns) per K row,
+// 4 K rows per 512-byte atom, 32-byte chunk j of K row k at chunk j ^ (k & 3).
+// A gathered row is two such 128-byte pieces, its 16-byte units copied straight
+// to their places.
 //
 // Complex product as two real products.  With A = Ar + i Ai (the two planes)
 // and the right-hand sides B stored as reals [k][2c + (0 re, 1 im)], the MMA
@@ -31,30 +34,53 @@
 // low 13 mantissa bits -- FP32 accumulation); then
 //   Re C(i, c) = Dr[i][2c] - Di[i][2c+1],  Im C(i, c) = Dr[i][2c+1] + Di[i][2c].
 //
-// Kernel: persistent, two CTAs per SM, tiles (front, 128-row tile, 32-column
-// chunk) taken in a fixed stride.  Warp roles:
-//   warp 0      bulk copies: lanes 0-3 the panel blocks, the right-hand-side
-//               rows into the stage's staging rows (one copy per run of
-//               rows that are contiguous in memory, else one per row; the
-//               update-row indices of the backward product looked up by
-//               the lanes first), one mbarrier transaction count
+// Kernel: one launch for both sweeps over the whole tree, two CTAs per SM.
+// Every CTA draws tiles (front, 128-row tile, 32-column chunk) from one list by
+// an atomic counter: the forward tiles, deepest level first, then the backward
+// ones, root level first, a level's tiles by subdomain and front, first
+// children before second ones.  What a tile waits for comes earlier in the
+// list, so it is done or being done by a running CTA whatever the number of
+// CTAs that run at the same time:
+//   - forward tile of a front: all forward tiles of its children, counted per
+//     front by the epilogues (release) and polled by the copy warp (acquire);
+//   - backward tile: all backward tiles of the parent (of the root: its own
+//     forward tiles), which closes the chain over everything else it reads.
+// The children add their update rows straight into the parent's pivot rows in
+// Y, the first child, then the second (whose epilogue waits for the first
+// child's count), so the sum has a fixed order; update rows that meet the
+// parent's update rows go through upd.  (With the two children next to each
+// other in the list the waits formed chains from CTA to CTA: 6.8 ms per
+// application of 32 columns on 402,444 tets.)
+// Why one launch: with a launch per level and direction (and one more for the
+// extend-add of the pivot rows) every level ended in a partly filled last wave
+// and began with the set-up of all CTAs; subdomains, whose levels are
+// independent of each other, now overlap across levels.  Measured: XX3.
+// Warp roles:
+//   warp 0      streams the panel blocks by bulk copies, which depend on no
+//               other tile
 //   warp 1      owns the tensor memory (2 x 128 columns: accumulators double
 //               buffered across tiles); one lane issues tcgen05.mma and commits
-//   warps 2-3   transpose the staging rows into the K-major B tile (shared
-//               memory only)
+//   warps 2-3   wait for a tile's dependencies and gather the right-hand-side
+//               rows into the B operand by 16-byte asynchronous copies (16 lanes
+//               a row).  The chain of a stage -- free, gathered, multiplied --
+//               sets its rate: with a K-major B, which took a transposition
+//               through shared memory between the two, the same launch ran
+//               XX4, with one bulk copy per run of contiguous rows XX5.
 //   warps 4-7   epilogue: tcgen05.ld, complex combine, D^{-1} scaling or
-//               extend-add of the children's update rows, global stores
-// Stages (2 x 48 KB per CTA, two CTAs per SM) form a ring shared by all tiles
-// of the CTA, so loads of the next tile overlap the products and the epilogue
-// of the current one; no
-// thread waits on device memory inside a stage except the copy lanes' index
-// lookups.  The right-hand-side rows move by 16-byte-aligned bulk copies, so
-// the engine needs an even number of columns (the solver falls back to the
-// mma.sync engine otherwise).
-// Every wait is bounded: on expiry the kernel records an error code, the
-// other roles stop at their next wait, and the CTA frees its tensor memory
-// and returns.
+//               extend-add, global stores, the front's count
+//   warp 8      draws the tiles, one ahead of warp 0 (a long tile does not hold
+//               back one that others wait for): descriptor into the ring,
+//               update-row indices into shared memory, the first part of the
+//               panel into L2
+// Stages (per CTA, two CTAs per SM) form a ring shared by all tiles of the CTA,
+// so loads of the next tile overlap the products and the epilogue of the
+// current one.  The rows are copied in units of 16 bytes, so the engine needs an
+// even number of columns.
+// Every wait is bounded: on expiry the kernel records an error code, the other
+// roles stop at their next wait, other CTAs at their next dependency wait, and
+// the CTA frees its tensor memory and returns.
 #include <algorithm>
+#include <mutex>
 
 #include "common.h"
 #include "kernels.h"
@@ -62,20 +88,27 @@
 namespace mwi {
 namespace {
 
-constexpr int kStages = 2;                  // stage ring per CTA (two CTAs per SM)
 constexpr int kCtasPerSm = 2;
+constexpr int kStages = 2;                  // stage ring per CTA
+constexpr int kKS = 4;                      // K steps of 8 per stage
+constexpr int kKRows = 8 * kKS;
+constexpr int kAStage = kKS * 8192;         // K steps x 16 groups of 8 M lines x 2 planes x 256 B
+constexpr int kBStage = kKRows * 256;       // two column groups x K rows x 128 B
+constexpr int kStage = kAStage + kBStage;
 constexpr int kUrCache = 1024;              // update-row indices of a backward tile kept in shared memory
-constexpr int kKS = 4;                      // K chunks of 8 per stage (K = 32)
-constexpr int kAStage = 32768;              // 4 K chunks x 16 groups of 8 M lines x 2 planes x 256 B
-constexpr int kBStage = 8192;               // 64 real columns x 32 K floats
-constexpr int kStage = kAStage + 2 * kBStage;  // + the staging rows [32][nc complex] of the copies
-constexpr int kThreads = 256;
+// tiles that can be under way in one CTA, each of one stage at least: index
+// buffers and descriptors (power of two) come round again after them
+constexpr int kSurBufs = kStages + 1;
+constexpr int kRing = 8;
+static_assert(kRing >= kStages + 3, "descriptor ring");
+constexpr int kThreads = 288;
 constexpr int kTmemCols = 256;
-constexpr int kSmemBytes = kStages * kStage + 1024 /* barriers */ + kUrCache * 4 + 1024 /* alignment */;
+constexpr int kSmemBytes =
+    kStages * kStage + 1024 /* barriers */ + kRing * 128 + kSurBufs * kUrCache * 4 + 1024 /* alignment */;
 static_assert(kSmemBytes * kCtasPerSm <= 228 * 1024 - 2048, "shared memory per SM");
 constexpr long long kWaitLimit = 1ll << 24;
-
-enum { kFwdT = 0, kBwdT = 1 };
+constexpr int kDepLimit = 1 << 22;          // polls of a dependency count (a few seconds)
+constexpr int kAheadSteps = 32;             // K steps of the next tile's panel fetched into L2
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -122,26 +155,27 @@ __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// shared-memory matrix descriptor of a K-major operand: start, leading /
-// stride byte offsets (>> 4; the leading offset is unused by swizzled K-major
-// layouts), version 1 (bit 46), layout type at bits 61-63 (2 = 128-byte
-// swizzle, 6 = 32-byte swizzle)
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t sbo, uint32_t layout) {
+// shared-memory matrix descriptor: start, leading and stride byte offsets (>> 4),
+// version 1 (bit 46), layout type at bits 61-63 (1 = 128-byte swizzle of 32-byte
+// atoms, 6 = 32-byte swizzle).  K-major: stride offset between groups of 8
+// lines, leading offset unused; MN-major: leading offset between groups of 32
+// columns, stride offset between groups of 4 K rows
+__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo, uint32_t layout) {
     uint64_t d = 0;
     d |= (uint64_t)((addr >> 4) & 0x3FFF);
-    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
     d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
     d |= (uint64_t)1 << 46;
     d |= (uint64_t)layout << 61;
     return d;
 }
-constexpr uint32_t kSw128 = 2, kSw32 = 6;
+constexpr uint32_t kSw128Base32 = 1, kSw32 = 6;
 
 // instruction descriptor of kind::tf32: D FP32 (bits 4-5 = 1), A and B TF32
-// (bits 7-9, 10-12 = 2), both K-major (bits 15, 16 = 0), N >> 3 at bits
-// 17-22, M >> 4 at bits 24-28
+// (bits 7-9, 10-12 = 2), A K-major (bit 15 = 0), B MN-major (bit 16 = 1),
+// N >> 3 at bits 17-22, M >> 4 at bits 24-28
 __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
-    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+    return (1u << 4) | (2u << 7) | (2u << 10) | (1u << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
@@ -171,6 +205,45 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+__device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+// 16 bytes global -> shared past L1, asynchronously (bytes = 0: zeros, nothing
+// is read); copies_arrive: this thread's arrival on the barrier once its copies
+// so far have landed
+__device__ __forceinline__ void copy16(uint32_t dst, const void* src, uint32_t bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void copies_arrive(uint32_t bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ int ld_acquire(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void red_release(int* p) {
+    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p) : "memory");
+}
+// bounded wait until *cnt >= target (one lane); false if the CTA aborts, another
+// CTA has reported an error or the limit expires
+__device__ __forceinline__ bool dep_wait(const int* cnt, int target, volatile int* abort_flag, int* err, int code) {
+    for (int it = 0; it < kDepLimit; ++it) {
+        if (ld_acquire(cnt) >= target) return true;
+        if (*abort_flag) return false;
+        if ((it & 63) == 63) {
+            if (ld_acquire(err)) {
+                *abort_flag = 1;
+                return false;
+            }
+        }
+        if (it > 64) __nanosleep(64);
+    }
+    *abort_flag = 1;
+    atomicExch(err, code);
+    return false;
+}
+
 // Tile geometry shared by every role.  Forward: M = front rows row0..
 // (row groups g0.., ng of them), K = pivots [0, min(p, row0 + 128)) in chunks
 // of 8.  Backward: M = pivots row0.. (pivot groups g0..), K = front rows from
@@ -178,24 +251,25 @@ __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.
 // chunks of a front's copy are cstride blocks apart.
 struct TcGeom {
     int p, f, row0, g0, ng, k0, nk, nst, cstride;
+    bool bwd;
 };
 
-template <int MODE>
-__device__ __forceinline__ TcGeom tc_geom(const TileDesc& d) {
+__device__ __forceinline__ TcGeom tc_geom(int p, int f, int row0, bool bwd) {
     TcGeom g;
-    g.p = d.p;
-    g.f = d.f;
-    g.row0 = d.row0;
-    const int F8 = (d.f + 7) >> 3, P8 = (d.p + 7) >> 3;
-    g.g0 = d.row0 >> 3;
-    if (MODE == kFwdT) {
+    g.p = p;
+    g.f = f;
+    g.row0 = row0;
+    g.bwd = bwd;
+    const int F8 = (f + 7) >> 3, P8 = (p + 7) >> 3;
+    g.g0 = row0 >> 3;
+    if (!bwd) {
         g.ng = min(16, F8 - g.g0);
         g.k0 = 0;
-        g.nk = (min(d.p, d.row0 + 128) + 7) >> 3;
+        g.nk = (min(p, row0 + 128) + 7) >> 3;
         g.cstride = F8;
     } else {
         g.ng = min(16, P8 - g.g0);
-        g.k0 = d.row0 >> 3;
+        g.k0 = row0 >> 3;
         g.nk = F8 - g.k0;
         g.cstride = P8;
     }
@@ -203,50 +277,74 @@ __device__ __forceinline__ TcGeom tc_geom(const TileDesc& d) {
     return g;
 }
 
-// number of the stage's 32 K rows that hold data (the rest of the B tile is zero)
-template <int MODE>
+// number of the stage's K rows that hold data (the rest of its last K step is zero)
 __device__ __forceinline__ int stage_rows(const TcGeom& G, int st) {
-    const int lim = MODE == kFwdT ? min(G.p, G.row0 + 128) - st * 32 : G.f - (G.row0 + st * 32);
-    return max(0, min(32, lim));
+    const int lim = !G.bwd ? min(G.p, G.row0 + 128) - st * kKRows : G.f - (G.row0 + st * kKRows);
+    return min(kKRows, lim);
 }
 
-template <int MODE>
+// backward tiles keep their update-row indices in shared memory, if they fit
+// beside the up to three that the copy's alignment brings along
+__device__ __forceinline__ bool indices_cached(const TcGeom& G) {
+    return G.bwd && G.f > G.p && G.f - G.p <= kUrCache - 3;
+}
+
+// a tile as the roles read it from the ring: the descriptor's words, then the
+// chunk's first column and whether there is a tile
+struct RingSlot {
+    TcTile d;
+    int c0, valid;
+    int pad[32 - sizeof(TcTile) / 4 - 2];
+};
+static_assert(sizeof(RingSlot) == 128 && sizeof(TcTile) % 4 == 0, "one descriptor per 128 bytes");
+constexpr int kTileWords = sizeof(TcTile) / 4;
+
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
-    const TileDesc* __restrict__ tiles, int ntiles, int nchunks, const int32_t* __restrict__ urows,
-    const int2* __restrict__ asm2, const float* __restrict__ wt, const float2* __restrict__ dinv,
-    float2* __restrict__ Y, float2* __restrict__ Z, float2* __restrict__ upd, int m, int* __restrict__ err) {
+    const TcTile* __restrict__ tiles, int ntiles, int nchunks, int* __restrict__ cnt,
+    const int32_t* __restrict__ urows, const int2* __restrict__ asm2, const int32_t* __restrict__ pdst,
+    const float* __restrict__ wt, const float2* __restrict__ dinv, float2* Y, float2* Z, float2* upd, int m,
+    int* err) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                            ~(uintptr_t)1023);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStage);
-    // bars: raw[kStages] (copies landed), full[kStages] (B tile ready), empty[kStages]
-    // (stage consumed), tfull[2], tempty[2]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * kStages + 4);
+    // bars: raw[kStages] (panel blocks landed), rows[kStages] (right-hand-side rows
+    // landed), empty[kStages] (stage consumed), tfull[2], tempty[2], tile[kRing]
+    // (descriptor written), sur[kSurBufs], begun (tile begun)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * kStages + 4 + kRing + kSurBufs + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    int32_t* sur = reinterpret_cast<int32_t*>(smem + kStages * kStage + 1024);  // copy warp's index cache
+    RingSlot* ring = reinterpret_cast<RingSlot*>(smem + kStages * kStage + 1024);
+    int32_t* sur = reinterpret_cast<int32_t*>(smem + kStages * kStage + 1024 + kRing * 128);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t sbase = smem_u32(smem);
     auto raw_bar = [&](int s) { return smem_u32(bars + s); };
-    auto full_bar = [&](int s) { return smem_u32(bars + kStages + s); };
+    auto rows_bar = [&](int s) { return smem_u32(bars + kStages + s); };
     auto empty_bar = [&](int s) { return smem_u32(bars + 2 * kStages + s); };
     auto tfull_bar = [&](int b) { return smem_u32(bars + 3 * kStages + b); };
     auto tempty_bar = [&](int b) { return smem_u32(bars + 3 * kStages + 2 + b); };
+    auto tile_bar = [&](int it) { return smem_u32(bars + 3 * kStages + 4 + (it & (kRing - 1))); };
+    auto tile_par = [&](int it) { return (uint32_t)(it / kRing) & 1; };
+    auto sur_bar = [&](int b) { return smem_u32(bars + 3 * kStages + 4 + kRing + b); };
+    const uint32_t begun_bar = smem_u32(bars + 3 * kStages + 4 + kRing + kSurBufs);
 
-    // stale shared memory must be finite: the MMA reads whole blocks, and the
-    // zero right-hand-side rows only cancel finite factor entries
+    // stale shared memory must be finite: the MMA reads whole 128-row groups of
+    // panel blocks, and the columns and rows without data go nowhere
     for (int i = threadIdx.x; i < kStages * kStage / 16; i += kThreads)
         reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
     fence_proxy_async();
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(raw_bar(s), 1);       // the copy lane, with the stage's transaction bytes
-            mbar_init(full_bar(s), 2);      // the 2 transpose warps
+            mbar_init(rows_bar(s), 64);     // the lanes of the gather warps
             mbar_init(empty_bar(s), 1);     // tcgen05.commit
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(tfull_bar(b), 1);
             mbar_init(tempty_bar(b), 4);    // the 4 epilogue warps
         }
+        for (int b = 0; b < kSurBufs; ++b) mbar_init(sur_bar(b), 1);
+        for (int b = 0; b < kRing; ++b) mbar_init(tile_bar(b), 1);
+        mbar_init(begun_bar, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -262,89 +360,45 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
     const int total = ntiles * nchunks;
 
     if (warp == 0) {
-        // ---------------- bulk copies: panel blocks (lane 0) and one
-        // right-hand-side row per lane into the stage's staging rows
+        // ---------------- panel blocks
         long long g = 0;
         bool ok = true;
-        for (int ti = blockIdx.x; ti < total && ok; ti += gridDim.x) {
-            const TileDesc d = tiles[ti / nchunks];
-            const TcGeom G = tc_geom<MODE>(d);
-            const int c0 = (ti % nchunks) * 32, nc = min(32, m - c0);
-            const uint32_t row_bytes = (uint32_t)nc * 8u;
-            const float* P = wt + d.a_off;
-            const int32_t* ur = urows + d.u_off;
-            // backward: the tile's update-row indices (at most kUrCache) into shared
-            // memory, one coalesced pass; the stages then look them up there
-            const int u = G.f - G.p;
-            const bool ur_cached = MODE == kBwdT && u <= kUrCache;
-            __syncwarp();
-            if (ur_cached) {
-                // eight loads in flight per lane before their stores
-                for (int j0 = 0; j0 < u; j0 += 256) {
-                    int v[8];
-#pragma unroll
-                    for (int t = 0; t < 8; ++t) {
-                        const int j = j0 + 32 * t + lane;
-                        v[t] = j < u ? ur[j] : 0;
-                    }
-#pragma unroll
-                    for (int t = 0; t < 8; ++t) {
-                        const int j = j0 + 32 * t + lane;
-                        if (j < u) sur[j] = v[t];
-                    }
-                }
-                __syncwarp();
-            }
+        for (int it = 0; ok; ++it) {
+            if (!(ok = mbar_wait(tile_bar(it), tile_par(it), abort_flag, err, 8))) break;
+            const RingSlot* slot = ring + (it & (kRing - 1));
+            if (!slot->valid) break;
+            const TcGeom G = tc_geom(slot->d.p, slot->d.f, slot->d.row0, slot->d.bwd != 0);
+            const float* P = wt + slot->d.a_off;
+            const uint32_t a_bytes = (uint32_t)G.ng * 512u;
             for (int st = 0; st < G.nst; ++st, ++g) {
                 const int s = (int)(g % kStages);
                 const uint32_t ph = (uint32_t)((g / kStages) & 1);
-                // the source row of this lane, looked up before the stage is free
-                const int nv = stage_rows<MODE>(G, st);
-                const float2* src = nullptr;
-                if (lane < nv) {
-                    if (MODE == kFwdT) {
-                        src = Y + (d.rowbase + st * 32 + lane) * m + c0;
-                    } else {
-                        const int i = G.row0 + st * 32 + lane;
-                        src = i < G.p ? Z + (d.rowbase + i) * m + c0
-                                      : Y + (d.sbase + (ur_cached ? sur[i - G.p] : ur[i - G.p])) * m + c0;
-                    }
-                }
-                if (lane == 0) ok = mbar_wait(empty_bar(s), ph ^ 1, abort_flag, err, 1);
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (!ok) break;
-                const uint32_t a_dst = sbase + s * kStage;
+                if (!(ok = mbar_wait(empty_bar(s), ph ^ 1, abort_flag, err, 1))) break;
                 const int k0 = G.k0 + st * kKS, nk = min(kKS, G.k0 + G.nk - k0);
-                const uint32_t a_bytes = (uint32_t)G.ng * 512u;
-                if (lane == 0) mbar_arrive_tx(raw_bar(s), a_bytes * nk + row_bytes * nv);
+                if (lane == 0) mbar_arrive_tx(raw_bar(s), a_bytes * nk);
                 __syncwarp();
                 if (lane < nk)
-                    bulk_g2s(a_dst + lane * 8192, P + ((int64_t)(k0 + lane) * G.cstride + G.g0) * 128, a_bytes,
-                             raw_bar(s));
-                // right-hand-side rows: with one column chunk (nc = m) consecutive rows are
-                // contiguous in memory, so each run of consecutive source rows moves as one
-                // copy (the forward pivot rows are one run; the backward rows a few)
-                const unsigned long long sa = reinterpret_cast<unsigned long long>(src);
-                const unsigned long long prev = __shfl_up_sync(0xffffffffu, sa, 1);
-                const bool lead = lane < nv && (nchunks > 1 || lane == 0 || sa != prev + row_bytes);
-                const unsigned leaders = __ballot_sync(0xffffffffu, lead);
-                if (lead) {
-                    const unsigned later = leaders & ~((2u << lane) - 1u);
-                    const int len = (later ? __ffs(later) - 1 : nv) - lane;
-                    bulk_g2s(a_dst + kAStage + kBStage + lane * row_bytes, src, row_bytes * (uint32_t)len, raw_bar(s));
-                }
+                    bulk_g2s(sbase + s * kStage + lane * 8192, P + ((int64_t)(k0 + lane) * G.cstride + G.g0) * 128,
+                             a_bytes, raw_bar(s));
+                if (st == 0 && lane == 0) mbar_arrive(begun_bar);
             }
         }
+        if (!ok && lane == 0)
+            // copies still in flight land before the CTA gives its shared memory back
+            for (long long q = g > kStages ? g - kStages : 0; q < g; ++q)
+                for (int it = 0; it < (1 << 12); ++it)
+                    if (mbar_try(raw_bar((int)(q % kStages)), (uint32_t)((q / kStages) & 1))) break;
     } else if (warp == 1) {
         // ---------------- tensor-core products
         if (lane == 0) {
             long long g = 0;
-            int it = 0;
             bool ok = true;
             constexpr uint32_t kIdesc = idesc_tf32(128, 64);
-            for (int ti = blockIdx.x; ti < total && ok; ti += gridDim.x, ++it) {
-                const TileDesc d = tiles[ti / nchunks];
-                const TcGeom G = tc_geom<MODE>(d);
+            for (int it = 0; ok; ++it) {
+                if (!mbar_wait(tile_bar(it), tile_par(it), abort_flag, err, 8)) break;
+                const RingSlot* slot = ring + (it & (kRing - 1));
+                if (!slot->valid) break;
+                const TcGeom G = tc_geom(slot->d.p, slot->d.f, slot->d.row0, slot->d.bwd != 0);
                 const int buf = it & 1;
                 if (!(ok = mbar_wait(tempty_bar(buf), ((it >> 1) & 1) ^ 1, abort_flag, err, 2))) break;
                 tc_fence_after();
@@ -352,16 +406,18 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                 for (int st = 0; st < G.nst; ++st, ++g) {
                     const int s = (int)(g % kStages);
                     const uint32_t ph = (uint32_t)((g / kStages) & 1);
-                    if (!(ok = mbar_wait(full_bar(s), ph, abort_flag, err, 3))) break;
+                    if (!(ok = mbar_wait(raw_bar(s), ph, abort_flag, err, 3))) break;
+                    if (!(ok = mbar_wait(rows_bar(s), ph, abort_flag, err, 4))) break;
+                    fence_proxy_async();
                     tc_fence_after();
                     const uint32_t a0 = sbase + s * kStage, b0 = a0 + kAStage;
                     const int nk = min(kKS, G.nk - st * kKS);
                     for (int c = 0; c < nk; ++c) {
-                        // B: 64 lines (real columns) of 128 B, K step c = bytes 32c of every line
-                        const uint64_t bd = smem_desc(b0 + c * 32, 1024, kSw128);
+                        // B: K step c = two 512-byte atoms in each of the two column groups
+                        const uint64_t bd = smem_desc(b0 + c * 1024, kKRows * 128, 512, kSw128Base32);
                         const uint32_t acc = (st > 0 || c > 0) ? 1u : 0u;
-                        mma_tf32(dr, smem_desc(a0 + c * 8192, 512, kSw32), bd, kIdesc, acc);
-                        mma_tf32(di, smem_desc(a0 + c * 8192 + 256, 512, kSw32), bd, kIdesc, acc);
+                        mma_tf32(dr, smem_desc(a0 + c * 8192, 16, 512, kSw32), bd, kIdesc, acc);
+                        mma_tf32(di, smem_desc(a0 + c * 8192 + 256, 16, 512, kSw32), bd, kIdesc, acc);
                     }
                     mma_commit(empty_bar(s));
                 }
@@ -370,79 +426,148 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             }
         }
     } else if (warp < 4) {
-        // ---------------- staging rows [32][nc complex] -> K-major B tile
-        // (line = real column, 32 K floats, 128-byte swizzle); thread: column
-        // `lane`, four groups of 4 rows
-        const int rg = warp - 2;
+        // ---------------- right-hand-side rows into the B operand: this warp's half
+        // of the stage's K rows
+        constexpr int kMine = kKRows / 4;  // row pairs of a stage per warp
+        const int seg = lane & 15, half = lane >> 4, first = (warp - 2) * (kKRows / 2) + half;
         long long g = 0;
+        int nsur = 0;
         bool ok = true;
-        for (int ti = blockIdx.x; ti < total && ok; ti += gridDim.x) {
-            const TileDesc d = tiles[ti / nchunks];
-            const TcGeom G = tc_geom<MODE>(d);
-            const int nc = min(32, m - (ti % nchunks) * 32);  // columns of the chunk (staging row length)
-            const bool cin = lane < nc;
+        for (int it = 0; ok; ++it) {
+            if (!mbar_wait(tile_bar(it), tile_par(it), abort_flag, err, 8)) break;
+            const RingSlot* slot = ring + (it & (kRing - 1));
+            if (!slot->valid) break;
+            const TcGeom G = tc_geom(slot->d.p, slot->d.f, slot->d.row0, slot->d.bwd != 0);
+            const int c0 = slot->c0, nc = min(32, m - c0);
+            // rows in units of 16 bytes from the first of this lane
+            const uint32_t ld = (uint32_t)m >> 1;
+            const float4* own = reinterpret_cast<const float4*>((G.bwd ? Z : Y) + slot->d.rowbase * m + c0) + seg;
+            const float4* anc = reinterpret_cast<const float4*>(Y + slot->d.sbase * m + c0) + seg;
+            const int32_t* iu = urows + slot->d.u_off;
+            const int kfirst = G.bwd ? G.row0 : 0;
+            if (indices_cached(G)) {
+                if (!(ok = mbar_wait(sur_bar(nsur % kSurBufs), (uint32_t)(nsur / kSurBufs) & 1, abort_flag, err, 6)))
+                    break;
+                iu = sur + (nsur % kSurBufs) * kUrCache + (slot->d.u_off & 3);
+                ++nsur;
+            }
+            // the rows are other tiles' results
+            if (lane < 2) {
+                const int dep = lane == 0 ? slot->d.dep0 : slot->d.dep1;
+                if (dep >= 0)
+                    ok = dep_wait(cnt + dep, (lane == 0 ? slot->d.need0 : slot->d.need1) * nchunks, abort_flag, err, 7);
+            }
+            if (!(ok = __all_sync(0xffffffffu, ok))) break;
             for (int st = 0; st < G.nst; ++st, ++g) {
                 const int s = (int)(g % kStages);
                 const uint32_t ph = (uint32_t)((g / kStages) & 1);
-                if (!(ok = mbar_wait(raw_bar(s), ph, abort_flag, err, 4))) break;
-                const int nv = stage_rows<MODE>(G, st);
-                unsigned char* B = smem + s * kStage + kAStage;
-                const float2* R = reinterpret_cast<const float2*>(B + kBStage);
+                const int nv = stage_rows(G, st);
+                const int nz = min(kKRows, (nv + 7) & ~7);  // rows that the products read
+                const uint32_t R = sbase + s * kStage + kAStage + (seg >> 3) * (kKRows * 128) + (seg & 1) * 16;
+                if (!(ok = mbar_wait(empty_bar(s), ph ^ 1, abort_flag, err, 1))) break;
+                if (seg < (nc >> 1)) {
+                    // all addresses before the copies, which the compiler keeps in order
+                    // with the index loads
+                    const float4* src[kMine];
 #pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    const int q = rg * 4 + h;  // rows 4q .. 4q+3
-                    float2 v[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int r = 4 * q + j;
-                        v[j] = (cin && r < nv) ? R[r * nc + lane] : make_float2(0.f, 0.f);
+                    for (int j = 0; j < kMine; ++j) {
+                        const int r = min(first + 2 * j, nv - 1);  // row of the stage
+                        const int k = kfirst + st * kKRows + r;
+                        const bool piv = !G.bwd || k < G.p;
+                        const uint32_t row = piv ? k : iu[k - G.p];
+                        src[j] = (piv ? own : anc) + (uint64_t)row * ld;
                     }
-                    const int n0 = 2 * lane;
-                    *reinterpret_cast<float4*>(B + (n0 >> 3) * 1024 + (n0 & 7) * 128 + ((q ^ (n0 & 7)) << 4)) =
-                        make_float4(v[0].x, v[1].x, v[2].x, v[3].x);
-                    const int n1 = n0 + 1;
-                    *reinterpret_cast<float4*>(B + (n1 >> 3) * 1024 + (n1 & 7) * 128 + ((q ^ (n1 & 7)) << 4)) =
-                        make_float4(v[0].y, v[1].y, v[2].y, v[3].y);
+#pragma unroll
+                    for (int j = 0; j < kMine; ++j) {
+                        const int r = first + 2 * j;
+                        if (r < nz)
+                            copy16(R + r * 128 + ((((seg & 7) >> 1) ^ (r & 3)) << 5), src[j], r < nv ? 16u : 0u);
+                    }
                 }
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(full_bar(s));
+                copies_arrive(rows_bar(s));
             }
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+    } else if (warp == 8) {
+        // ---------------- tiles.  A ring slot or an index buffer is free when it
+        // comes round again: tile i is drawn after the first panel blocks of tile
+        // i - 1 are under way, i.e. after the products of the stage kStages before,
+        // which is of tile i - 1 - kStages or later: that tile's rows are gathered,
+        // and its accumulator waited for the epilogue of the tile two before.
+        int nsur = 0;  // index buffers filled so far
+        bool ok = true;
+        for (int it = 0;; ++it) {
+            if (it > 0 && !(ok = mbar_wait(begun_bar, (uint32_t)(it - 1) & 1, abort_flag, err, 10))) break;
+            const int tk = __shfl_sync(0xffffffffu, lane == 0 ? atomicAdd(cnt, 1) : 0, 0);
+            const int ti = tk / nchunks;
+            RingSlot* slot = ring + (it & (kRing - 1));
+            uint32_t w = 0;
+            if (lane < kTileWords) w = tk < total ? reinterpret_cast<const uint32_t*>(tiles + ti)[lane] : 0u;
+            else if (lane == kTileWords) w = (uint32_t)((tk - ti * nchunks) * 32);
+            else if (lane == kTileWords + 1) w = tk < total ? 1u : 0u;
+            reinterpret_cast<uint32_t*>(slot)[lane] = w;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(tile_bar(it));
+            if (tk >= total) break;
+            const TcGeom G = tc_geom(slot->d.p, slot->d.f, slot->d.row0, slot->d.bwd != 0);
+            if (indices_cached(G) && lane == 0) {
+                // one bulk copy, the start rounded down to 16 bytes (the list is padded at its end)
+                const int off = (int)(slot->d.u_off & 3);
+                const uint32_t bar = sur_bar(nsur % kSurBufs), bytes = (uint32_t)((G.f - G.p + off + 3) / 4) * 16u;
+                fence_proxy_async();
+                mbar_arrive_tx(bar, bytes);
+                bulk_g2s(smem_u32(sur + (nsur % kSurBufs) * kUrCache), urows + (slot->d.u_off - off), bytes, bar);
+            }
+            nsur += indices_cached(G) ? 1 : 0;
+            if (lane < min(G.nk, kAheadSteps))
+                l2_prefetch(wt + slot->d.a_off + ((int64_t)(G.k0 + lane) * G.cstride + G.g0) * 128,
+                            (uint32_t)G.ng * 512u);
+        }
+        if (!ok && lane == 0)
+            for (int q = max(0, nsur - kSurBufs); q < nsur; ++q)
+                for (int it = 0; it < (1 << 12); ++it)
+                    if (mbar_try(sur_bar(q % kSurBufs), (uint32_t)(q / kSurBufs) & 1)) break;
     } else {
         // ---------------- epilogue
         const int lg = warp & 3;  // tensor-memory lane group of this warp
         const int i = lg * 32 + lane;
-        int it = 0;
         bool ok = true;
-        for (int ti = blockIdx.x; ti < total && ok; ti += gridDim.x, ++it) {
-            const TileDesc d = tiles[ti / nchunks];
-            const int c0 = (ti % nchunks) * 32;
+        for (int it = 0; ok; ++it) {
+            if (!mbar_wait(tile_bar(it), tile_par(it), abort_flag, err, 8)) break;
+            const RingSlot* slot = ring + (it & (kRing - 1));
+            if (!slot->valid) break;
+            const TcTile d = slot->d;
+            const bool bwd = d.bwd != 0;
+            const int c0 = slot->c0, nc = min(32, m - c0);
             const int buf = it & 1;
             // loads that do not depend on the product, issued before waiting for it
             const int gi = d.row0 + i;
             float2 dv = make_float2(0.f, 0.f);
             int2 src = make_int2(-1, -1);
-            if (MODE == kFwdT) {
-                if (gi < d.p) dv = dinv[d.rowbase + gi];
-                else if (gi < d.f) src = asm2[d.asm_base + gi];
+            float2* dst = nullptr;
+            bool add = false;  // dst holds rows to add to: a pivot row of the parent
+            if (gi < d.p) {
+                if (!bwd) dv = dinv[d.rowbase + gi];
+                dst = (bwd ? Y : Z) + (d.rowbase + gi) * m + c0;
+            } else if (!bwd && gi < d.f) {
+                src = asm2[d.asm_base + gi];
+                const int pd = pdst[d.upd_row + gi - d.p];
+                add = pd >= 0;
+                dst = add ? Y + (int64_t)pd * m + c0 : upd + (d.upd_row + gi - d.p) * m + c0;
+            }
+            if (d.sib >= 0 && __any_sync(0xffffffffu, add)) {
+                // the second child adds to the parent's rows after the first
+                if (lane == 0) ok = dep_wait(cnt + d.sib, d.needs * nchunks, abort_flag, err, 9);
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                if (!ok) break;
             }
             if (!(ok = mbar_wait(tfull_bar(buf), (it >> 1) & 1, abort_flag, err, 5))) break;
             tc_fence_after();
             const uint32_t t0 = tmem + ((uint32_t)(lg * 32) << 16) + buf * 128;
-            const int nc = min(32, m - c0);
-            float2* dst = nullptr;
-            if (MODE == kBwdT) {
-                if (gi < d.p) dst = Y + (d.rowbase + gi) * m + c0;
-            } else if (gi < d.p) {
-                dst = Z + (d.rowbase + gi) * m + c0;
-            } else if (gi < d.f) {
-                dst = upd + (d.upd_row + gi - d.p) * m + c0;
-            }
-            const bool vec = nc == 32 && (m & 1) == 0;
             // two halves of 16 complex columns: tensor-memory loads, combine,
-            // D^{-1} or the children's rows, stores; the accumulator is released
-            // once the second half is in registers
+            // D^{-1} or the rows to add, stores; the accumulator is released
+            // once the second half is in registers.  Rows that other tiles of
+            // this launch have written are read past L1.
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 float o[32];
@@ -462,52 +587,41 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tempty_bar(buf));
                 }
-                if (!dst) continue;
                 const int cb = 16 * h;  // first complex column of the half
-                if (MODE == kFwdT && gi < d.p) {
+                if (!dst || cb >= nc) continue;
+                if (gi < d.p && !bwd) {
 #pragma unroll
                     for (int q = 0; q < 16; ++q) {
                         const float re = o[2 * q], im = o[2 * q + 1];
                         o[2 * q] = re * dv.x - im * dv.y;
                         o[2 * q + 1] = re * dv.y + im * dv.x;
                     }
-                } else if (MODE == kFwdT) {
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        const int sr = k ? src.y : src.x;
-                        if (sr < 0) continue;
-                        const float2* a = upd + (int64_t)sr * m + c0 + cb;
-                        if (vec) {
-#pragma unroll
-                            for (int q = 0; q < 8; ++q) {
-                                const float4 v = reinterpret_cast<const float4*>(a)[q];
-                                o[4 * q] += v.x;
-                                o[4 * q + 1] += v.y;
-                                o[4 * q + 2] += v.z;
-                                o[4 * q + 3] += v.w;
-                            }
-                        } else {
-#pragma unroll
-                            for (int q = 0; q < 16; ++q)
-                                if (cb + q < nc) {
-                                    const float2 v = a[q];
-                                    o[2 * q] += v.x;
-                                    o[2 * q + 1] += v.y;
-                                }
-                        }
-                    }
                 }
-                if (vec) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const float2* a = k == 2 ? (add ? dst + cb : nullptr)
+                                             : ((k ? src.y : src.x) >= 0
+                                                    ? upd + (int64_t)(k ? src.y : src.x) * m + c0 + cb
+                                                    : nullptr);
+                    if (!a) continue;
 #pragma unroll
                     for (int q = 0; q < 8; ++q)
+                        if (cb + 2 * q < nc) {
+                            const float4 v = __ldcg(reinterpret_cast<const float4*>(a) + q);
+                            o[4 * q] += v.x;
+                            o[4 * q + 1] += v.y;
+                            o[4 * q + 2] += v.z;
+                            o[4 * q + 3] += v.w;
+                        }
+                }
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (cb + 2 * q < nc)
                         reinterpret_cast<float4*>(dst + cb)[q] =
                             make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        if (cb + q < nc) dst[cb + q] = make_float2(o[2 * q], o[2 * q + 1]);
-                }
             }
+            __syncwarp();
+            if (lane == 0) red_release(cnt + d.cnt);
         }
     }
     tc_fence_before();
@@ -577,31 +691,21 @@ int sweep_tc_ctas() {
     return n;
 }
 
-template <int MODE>
-static void launch_tc(const TileDesc* tiles, int64_t ntiles, int m, const int32_t* urows, const int2* asm2,
-                      const float* wt, const float2* dinv, float2* Y, float2* Z, float2* upd, int* err,
-                      cudaStream_t st) {
-    static bool attr = false;
-    if (!attr) {
-        MWI_CUDA(cudaFuncSetAttribute(sweep_tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      kSmemBytes));
-        attr = true;
-    }
+// both sweeps; cnt holds F.tc_counts() zeros
+void sweep_tc_solve(const FrontsDev& F, int m, const float* wt, const float2* dinv, float2* Y, float2* Z,
+                    float2* upd, int* cnt, int* err, cudaStream_t st) {
+    static std::once_flag attr;
+    std::call_once(attr, [] {
+        MWI_CUDA(cudaFuncSetAttribute(sweep_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+    });
     const int nchunks = (m + 31) / 32;
-    const int64_t total = ntiles * nchunks;
+    const int64_t total = F.tc_ntiles * nchunks;
+    MWI_REQUIRE(total + 2 * sweep_tc_ctas() < ((int64_t)1 << 31), MWI_EINVAL, "too many sweep tiles");
+    if (total <= 0) return;
     const int grid = (int)std::min<int64_t>(total, sweep_tc_ctas());
-    sweep_tc_kernel<MODE><<<grid, kThreads, kSmemBytes, st>>>(tiles, (int)ntiles, nchunks, urows, asm2, wt, dinv, Y,
-                                                              Z, upd, m, err);
+    sweep_tc_kernel<<<grid, kThreads, kSmemBytes, st>>>(F.tc_tiles.p, (int)F.tc_ntiles, nchunks, cnt, F.urows.p,
+                                                        F.asm2.p, F.pdst.p, wt, dinv, Y, Z, upd, m, err);
     MWI_CHECK_LAUNCH();
-}
-
-void sweep_tc_level(bool backward, const TileDesc* tiles, int64_t ntiles, int m, const int32_t* urows,
-                    const int2* asm2, const float* wt, const float2* dinv, float2* Y, float2* Z, float2* upd,
-                    int* err, cudaStream_t st) {
-    if (ntiles <= 0) return;
-    MWI_REQUIRE(ntiles * ((m + 31) / 32) < ((int64_t)1 << 31), MWI_EINVAL, "too many sweep tiles");
-    if (backward) launch_tc<kBwdT>(tiles, ntiles, m, urows, asm2, wt, dinv, Y, Z, upd, err, st);
-    else launch_tc<kFwdT>(tiles, ntiles, m, urows, asm2, wt, dinv, Y, Z, upd, err, st);
 }
 
 }  // namespace mwi
