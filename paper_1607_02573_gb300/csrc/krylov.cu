@@ -240,73 +240,141 @@ __global__ void convert_kernel(int64_t nm, const A* __restrict__ a, B* __restric
     b[e].y = a[e].y;
 }
 
-// Per column c: store the Hessenberg column k (h[0..k], hnorm), apply the
-// previous rotations, form the new one, update g, decide convergence.
+// The small per-column kernels below run one warp per column.  Their chains of
+// dependent FP64 operations bound them: with one thread per column and a global
+// load in every link a step's kernel took 27 us over 11 steps and the back
+// substitution 55 us (24 steps: 55 and 200 us), more than anything else of a
+// step on a small problem.  Lanes now hold 32 entries at a time and only the
+// recurrences are serial: 15 and 17 us (24 steps: 24 and 33 us).
+
+__device__ __forceinline__ double2 shfl2(double2 v, int lane) {
+    return make_double2(__shfl_sync(0xffffffffu, v.x, lane), __shfl_sync(0xffffffffu, v.y, lane));
+}
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ double2 warp_sum(double2 v) { return make_double2(warp_sum(v.x), warp_sum(v.y)); }
+
+// Rotations 0..j-1 of column c applied to a Hessenberg column with entries
+// entry(0..j) (row i of entry is asked for by lane i % 32); row i < j of the
+// rotated column goes to out(i, value), row j is returned to every lane.
+template <typename Entry, typename Out>
+__device__ __forceinline__ double2 rotate_column(int j, int m, int c, const double2* cs, const double2* sn,
+                                                 Entry entry, Out out) {
+    const int lane = threadIdx.x & 31;
+    double2 t = entry(0);
+    for (int base = 0; base < j; base += 32) {
+        const int i = base + lane;
+        double2 ci = make_double2(1.0, 0.0), si = make_double2(0.0, 0.0), h = si, u = si, mine = si;
+        if (i < j) {
+            ci = cs[i * m + c];
+            si = sn[i * m + c];
+            h = entry(i + 1);
+            u = cmul(cconj(ci), h);
+        }
+        const int nq = min(32, j - base);
+        for (int q = 0; q < nq; ++q) {
+            if (lane == q) mine = t;
+            t = csub(shfl2(u, q), cmul(cconj(shfl2(si, q)), t));
+        }
+        if (i < j) out(i, cadd(cmul(ci, mine), cmul(si, h)));
+    }
+    return t;
+}
+
+// the rotation that clears b against a, rows j and j + 1 of the column's
+// factor R and of g (lane 0 writes); returns g's new last entry
+__device__ __forceinline__ double2 new_rotation(int j, int m, int c, double2 a, double2 b, double2* Hj, double2* cs,
+                                                double2* sn, double2* g) {
+    const double den = sqrt(cabs2(a) + cabs2(b));
+    double2 cj, sj;
+    if (den > 0.0) { cj = cscale(cconj(a), 1.0 / den); sj = cscale(cconj(b), 1.0 / den); }
+    else { cj = make_double2(1.0, 0.0); sj = make_double2(0.0, 0.0); }
+    const double2 gj = g[j * m + c];
+    const double2 gn = cscale(cmul(cconj(sj), gj), -1.0);
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) {
+        cs[j * m + c] = cj;
+        sn[j * m + c] = sj;
+        Hj[j * m + c] = make_double2(den, 0.0);
+        Hj[(j + 1) * m + c] = make_double2(0.0, 0.0);
+        g[(j + 1) * m + c] = gn;
+        g[j * m + c] = cmul(cj, gj);
+    }
+    __syncwarp();
+    return gn;
+}
+
+// Per column c: rotate the Hessenberg column k (h[0..k], hnorm) by the previous
+// rotations, form the new one, update g, decide convergence.
 __global__ void arnoldi_kernel(int m, int k, int restart, const double2* __restrict__ h,
-                               const double* __restrict__ hnorm2, double2* __restrict__ H,
-                               double2* __restrict__ cs, double2* __restrict__ sn, double2* __restrict__ g,
-                               int* __restrict__ active, int* __restrict__ kcol, const double* __restrict__ tol,
-                               double* __restrict__ resid, double* __restrict__ inv_norm, int* __restrict__ n_active,
-                               float2* __restrict__ inv_df) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= m) return;
+                               const double* __restrict__ hnorm2, double2* __restrict__ H, double2* cs, double2* sn,
+                               double2* g, int* __restrict__ active, int* __restrict__ kcol,
+                               const double* __restrict__ tol, double* __restrict__ resid,
+                               double* __restrict__ inv_norm, int* __restrict__ n_active) {
+    const int c = blockIdx.x, lane = threadIdx.x;
     if (!active[c]) {
-        inv_norm[c] = 0.0;
-        if (inv_df) inv_df[c] = make_float2(0.f, 0.f);
+        if (lane == 0) inv_norm[c] = 0.0;
         return;
     }
     double2* Hk = H + (int64_t)k * (restart + 1) * m;
-    for (int i = 0; i <= k; ++i) Hk[i * m + c] = h[i * m + c];
     const double hn = sqrt(fmax(hnorm2[c], 0.0));
-    Hk[(k + 1) * m + c] = make_double2(hn, 0.0);
-    for (int i = 0; i < k; ++i) {
-        double2 ci = cs[i * m + c], si = sn[i * m + c];
-        double2 a = Hk[i * m + c], b = Hk[(i + 1) * m + c];
-        Hk[i * m + c] = cadd(cmul(ci, a), cmul(si, b));
-        Hk[(i + 1) * m + c] = csub(cmul(cconj(ci), b), cmul(cconj(si), a));
+    const double2 a = rotate_column(
+        k, m, c, cs, sn, [&](int i) { return h[i * m + c]; }, [&](int i, double2 v) { Hk[i * m + c] = v; });
+    const double2 gn = new_rotation(k, m, c, a, make_double2(hn, 0.0), Hk, cs, sn, g);
+    if (lane == 0) {
+        kcol[c] = k + 1;
+        const double rr = sqrt(cabs2(gn));
+        resid[c] = rr;
+        inv_norm[c] = hn > 0.0 ? 1.0 / hn : 0.0;
+        if (rr <= tol[c] || hn == 0.0 || !(rr == rr)) active[c] = 0;
+        else atomicAdd(n_active, 1);
     }
-    double2 a = Hk[k * m + c], b = Hk[(k + 1) * m + c];
-    double den = sqrt(cabs2(a) + cabs2(b));
-    double2 ck, sk;
-    if (den > 0.0) { ck = cscale(cconj(a), 1.0 / den); sk = cscale(cconj(b), 1.0 / den); }
-    else { ck = make_double2(1.0, 0.0); sk = make_double2(0.0, 0.0); }
-    cs[k * m + c] = ck;
-    sn[k * m + c] = sk;
-    Hk[k * m + c] = make_double2(den, 0.0);
-    Hk[(k + 1) * m + c] = make_double2(0.0, 0.0);
-    double2 gk = g[k * m + c];
-    g[(k + 1) * m + c] = cscale(cmul(cconj(sk), gk), -1.0);
-    g[k * m + c] = cmul(ck, gk);
-    kcol[c] = k + 1;
-    const double rr = sqrt(cabs2(g[(k + 1) * m + c]));
-    resid[c] = rr;
-    inv_norm[c] = hn > 0.0 ? 1.0 / hn : 0.0;
-    if (inv_df) inv_df[c] = df_split(inv_norm[c]);
-    if (rr <= tol[c] || hn == 0.0 || !(rr == rr)) active[c] = 0;
-    else atomicAdd(n_active, 1);
 }
 
-// y = R^{-1} g per column (R = rotated Hessenberg, kcol[c] columns)
+// y = R^{-1} g per column (R = rotated Hessenberg, kcol[c] columns), by columns
+// of R: the right-hand side sits in shared memory (or, beyond its size, in y)
 // ydf (optional) receives y as double-floats (re hi, re lo, im hi, im lo)
-__global__ void lsq_kernel(int m, int restart, const double2* __restrict__ H, const double2* __restrict__ g,
-                           const int* __restrict__ kcol, double2* __restrict__ y, float4* __restrict__ ydf) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= m) return;
+__global__ void lsq_kernel(int m, int restart, int in_smem, const double2* __restrict__ H,
+                           const double2* __restrict__ g, const int* __restrict__ kcol, double2* y,
+                           float4* __restrict__ ydf) {
+    extern __shared__ double2 lsq_smem[];
+    const int c = blockIdx.x, lane = threadIdx.x;
+    double2* w = in_smem ? lsq_smem : y + c;
+    const int ws = in_smem ? 1 : m;
     const int kk = kcol[c];
-    for (int i = kk; i < restart; ++i) y[i * m + c] = make_double2(0.0, 0.0);
-    for (int i = kk - 1; i >= 0; --i) {
-        double2 s = g[i * m + c];
-        for (int j = i + 1; j < kk; ++j)
-            s = csub(s, cmul(H[((int64_t)j * (restart + 1) + i) * m + c], y[j * m + c]));
-        double2 d = H[((int64_t)i * (restart + 1) + i) * m + c];
-        y[i * m + c] = (d.x == 0.0 && d.y == 0.0) ? make_double2(0.0, 0.0) : cdiv(s, d);
+    for (int i = lane; i < restart; i += 32) {
+        if (i < kk) w[i * (int64_t)ws] = g[i * m + c];
+        else y[i * (int64_t)m + c] = make_double2(0.0, 0.0);
     }
-    if (ydf)
-        for (int i = 0; i < restart; ++i) {
-            const double2 v = y[i * m + c];
+    __syncwarp();
+    auto R = [&](int r, int i) { return H[((int64_t)i * (restart + 1) + r) * m + c]; };
+    double2 d = kk > 0 ? R(kk - 1, kk - 1) : make_double2(0.0, 0.0);
+    double2 r0 = lane < kk - 1 ? R(lane, kk - 1) : make_double2(0.0, 0.0);
+    for (int i = kk - 1; i >= 0; --i) {
+        // the next column's entries on their way while this one's quotient is formed
+        const double2 dn = i > 0 ? R(i - 1, i - 1) : d;
+        const double2 rn = lane < i - 1 ? R(lane, i - 1) : r0;
+        const double2 s = w[i * (int64_t)ws];
+        const double2 yi = (d.x == 0.0 && d.y == 0.0) ? make_double2(0.0, 0.0) : cdiv(s, d);
+        __syncwarp();
+        for (int r = lane; r < i; r += 32)
+            w[r * (int64_t)ws] = csub(w[r * (int64_t)ws], cmul(r == lane ? r0 : R(r, i), yi));
+        if (lane == 0) w[i * (int64_t)ws] = yi;
+        __syncwarp();
+        d = dn;
+        r0 = rn;
+    }
+    for (int i = lane; i < restart; i += 32) {
+        const double2 v = i < kk ? w[i * (int64_t)ws] : make_double2(0.0, 0.0);
+        if (in_smem && i < kk) y[i * (int64_t)m + c] = v;
+        if (ydf) {
             const float2 a = df_split(v.x), b = df_split(v.y);
-            ydf[i * m + c] = make_float4(a.x, a.y, b.x, b.y);
+            ydf[i * (int64_t)m + c] = make_float4(a.x, a.y, b.x, b.y);
         }
+    }
 }
 
 // start of a cycle: g = (beta, 0, ...), inv = 1/beta, active = beta > tol
@@ -648,114 +716,89 @@ __global__ void __launch_bounds__(256) dots2_kernel(int64_t n, int m, int nq, co
 // without reorthogonalisation, which leaves the Arnoldi relation exact.
 __device__ __forceinline__ double2 conjmul(double2 a, double2 b) { return cmul(cconj(a), b); }
 
-__device__ void finalize_column(int m, int c, int j, int restart, double2* __restrict__ Hj,
-                                double2* __restrict__ cs, double2* __restrict__ sn, double2* __restrict__ g) {
-    for (int i = 0; i < j; ++i) {
-        const double2 ci = cs[i * m + c], si = sn[i * m + c];
-        const double2 a = Hj[i * m + c], b = Hj[(i + 1) * m + c];
-        Hj[i * m + c] = cadd(cmul(ci, a), cmul(si, b));
-        Hj[(i + 1) * m + c] = csub(cmul(cconj(ci), b), cmul(cconj(si), a));
-    }
-    const double2 a = Hj[j * m + c], b = Hj[(j + 1) * m + c];
-    const double den = sqrt(cabs2(a) + cabs2(b));
-    double2 cj, sj;
-    if (den > 0.0) { cj = cscale(cconj(a), 1.0 / den); sj = cscale(cconj(b), 1.0 / den); }
-    else { cj = make_double2(1.0, 0.0); sj = make_double2(0.0, 0.0); }
-    cs[j * m + c] = cj;
-    sn[j * m + c] = sj;
-    Hj[j * m + c] = make_double2(den, 0.0);
-    Hj[(j + 1) * m + c] = make_double2(0.0, 0.0);
-    const double2 gj = g[j * m + c];
-    g[(j + 1) * m + c] = cscale(cmul(cconj(sj), gj), -1.0);
-    g[j * m + c] = cmul(cj, gj);
-    (void)restart;
-}
-
 __device__ __forceinline__ float4 df4(double2 v) {
     const float2 a = df_split(v.x), b = df_split(v.y);
     return make_float4(a.x, a.y, b.x, b.y);
 }
 
 __global__ void arnoldi_dcgs_kernel(int m, int k, int restart, int last, const double2* __restrict__ dots,
-                                    double2* __restrict__ H, double2* __restrict__ Hp, double2* __restrict__ cs,
-                                    double2* __restrict__ sn, double2* __restrict__ g, int* __restrict__ active,
-                                    int* __restrict__ kcol, const double* __restrict__ tol,
+                                    double2* H, double2* Hp, double2* cs, double2* sn, double2* g,
+                                    int* __restrict__ active, int* __restrict__ kcol, const double* __restrict__ tol,
                                     double* __restrict__ resid, double* __restrict__ rho,
                                     int* __restrict__ n_active, float4* __restrict__ coefQ,
                                     float4* __restrict__ coefW, float4* __restrict__ scal) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= m) return;
-    const int nq = k, nout = 2 * nq + 3;
+    const int c = blockIdx.x, lane = threadIdx.x;
+    const int nq = k;
     const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
     if (!active[c]) {
-        for (int i = 0; i < nq; ++i) coefQ[i * m + c] = coefW[i * m + c] = z4;
-        scal[c] = scal[m + c] = z4;
+        for (int i = lane; i < nq; i += 32) coefQ[i * m + c] = coefW[i * m + c] = z4;
+        if (lane == 0) scal[c] = scal[m + c] = z4;
         return;
     }
-    const double2* a = dots;               // a_i = conj(q_i) v_k
-    const double2* b = dots + nq * m;      // b_i = conj(q_i) w
+    const double2* a = dots + c;           // a_i = conj(q_i) v_k
+    const double2* b = dots + nq * m + c;  // b_i = conj(q_i) w
     const double gam = dots[(2 * nq) * m + c].x;
     const double2 del = dots[(2 * nq + 1) * m + c];
     const double om = dots[(2 * nq + 2) * m + c].x;
+    // |a|^2, |b|^2 and q_k^H w's a^H b
+    double a2 = 0.0, b2 = 0.0;
+    double2 ab = make_double2(0.0, 0.0);
+    for (int i = lane; i < nq; i += 32) {
+        const double2 ai = a[i * m], bi = b[i * m];
+        a2 += cabs2(ai);
+        b2 += cabs2(bi);
+        ab = cadd(ab, conjmul(ai, bi));
+    }
+    a2 = warp_sum(a2);
+    b2 = warp_sum(b2);
+    ab = warp_sum(ab);
     double nu = 1.0;
     if (k > 0) {
-        double a2 = 0.0;
-        for (int i = 0; i < nq; ++i) a2 += cabs2(a[i * m + c]);
         nu = sqrt(fmax(gam - a2, 1e-30 * fmax(gam, 1e-300)));
         // column k-1: v_k = Q a + nu q_k, so h(i, k-1) += rho_{k-1} a_i and h(k, k-1) = rho_{k-1} nu
         const double r1 = rho[c];
         double2* Hc = H + (int64_t)(k - 1) * (restart + 1) * m;
-        const double2* Pc = Hp;
-        for (int i = 0; i < k; ++i) Hc[i * m + c] = cadd(Pc[i * m + c], cscale(a[i * m + c], r1));
-        Hc[k * m + c] = make_double2(r1 * nu, 0.0);
-        finalize_column(m, c, k - 1, restart, Hc, cs, sn, g);
+        const double2 t = rotate_column(
+            k - 1, m, c, cs, sn, [&](int i) { return cadd(Hp[i * m + c], cscale(a[i * m], r1)); },
+            [&](int i, double2 v) { Hc[i * m + c] = v; });
+        new_rotation(k - 1, m, c, t, make_double2(r1 * nu, 0.0), Hc, cs, sn, g);
     }
     // q_k^H w and the projected w's norm
-    double2 ab = make_double2(0.0, 0.0);
-    double b2 = 0.0;
-    for (int i = 0; i < nq; ++i) {
-        ab = cadd(ab, conjmul(a[i * m + c], b[i * m + c]));
-        b2 += cabs2(b[i * m + c]);
-    }
     const double2 ck = cscale(csub(del, ab), 1.0 / nu);
     const double rk = sqrt(fmax(om - b2 - cabs2(ck), 1e-14 * om));
-    // provisional column k: (b_0 .. b_{k-1}, c_k, rho_k)
-    for (int i = 0; i < nq; ++i) Hp[i * m + c] = b[i * m + c];
-    Hp[k * m + c] = ck;
-    Hp[(k + 1) * m + c] = make_double2(rk, 0.0);
-    // its rotated entry k (rotations 0..k-1), then the provisional residual
-    double2 t = nq > 0 ? b[c] : ck;
-    for (int i = 0; i < k; ++i) {
-        const double2 nxt = i + 1 < k ? b[(i + 1) * m + c] : ck;
-        const double2 ci = cs[i * m + c], si = sn[i * m + c];
-        t = csub(cmul(cconj(ci), nxt), cmul(cconj(si), t));
-    }
+    // provisional column k: (b_0 .. b_{k-1}, c_k, rho_k); its rotated entry k (rotations
+    // 0..k-1), then the provisional residual
+    auto col = [&](int i) { return i < k ? b[i * m] : ck; };
+    const double2 t = rotate_column(k, m, c, cs, sn, col, [](int, double2) {});
     const double den = sqrt(cabs2(t) + rk * rk);
     const double rr = den > 0.0 ? rk / den * sqrt(cabs2(g[k * m + c])) : 0.0;
-    resid[c] = rr;
-    rho[c] = rk;
+    for (int i = lane; i <= k; i += 32) Hp[i * m + c] = col(i);
     const bool stop = rr <= tol[c] || !(rr == rr) || rk == 0.0 || last;
     if (stop) {
         double2* Hc = H + (int64_t)k * (restart + 1) * m;
-        for (int i = 0; i <= k + 1; ++i) Hc[i * m + c] = Hp[i * m + c];
-        finalize_column(m, c, k, restart, Hc, cs, sn, g);
-        kcol[c] = k + 1;
-        if (!last) active[c] = 0;
-        else if (!(rr <= tol[c])) atomicAdd(n_active, 1);
-    } else {
-        kcol[c] = k;
-        atomicAdd(n_active, 1);
+        rotate_column(k, m, c, cs, sn, col, [&](int i, double2 v) { Hc[i * m + c] = v; });
+        new_rotation(k, m, c, t, make_double2(rk, 0.0), Hc, cs, sn, g);
+    }
+    if (lane == 0) {
+        Hp[(k + 1) * m + c] = make_double2(rk, 0.0);
+        resid[c] = rr;
+        rho[c] = rk;
+        kcol[c] = stop ? k + 1 : k;
+        if (stop && !last) active[c] = 0;
+        else if (!stop || !(rr <= tol[c])) atomicAdd(n_active, 1);
     }
     // fused update: q_k = v_k / nu - sum_i q_i a_i / nu;
     // v_{k+1} = w / rho_k - sum_i q_i (b_i - a_i c_k / nu) / rho_k - v_k c_k / (nu rho_k)
     const double inu = 1.0 / nu, irk = 1.0 / rk;
-    for (int i = 0; i < nq; ++i) {
-        const double2 ai = a[i * m + c];
+    for (int i = lane; i < nq; i += 32) {
+        const double2 ai = a[i * m];
         coefQ[i * m + c] = df4(cscale(ai, -inu));
-        coefW[i * m + c] = df4(cscale(csub(b[i * m + c], cscale(cmul(ai, ck), inu)), -irk));
+        coefW[i * m + c] = df4(cscale(csub(b[i * m], cscale(cmul(ai, ck), inu)), -irk));
     }
-    scal[c] = df4(make_double2(k > 0 ? inu : 1.0, irk));         // (1 / nu, 1 / rho_k) as reals
-    scal[m + c] = df4(cscale(ck, -inu * irk));                     // -c_k / (nu rho_k)
+    if (lane == 0) {
+        scal[c] = df4(make_double2(k > 0 ? inu : 1.0, irk));  // (1 / nu, 1 / rho_k) as reals
+        scal[m + c] = df4(cscale(ck, -inu * irk));            // -c_k / (nu rho_k)
+    }
 }
 
 // q_k (into V slot k, when k > 0) and v_{k+1} (into V slot k + 1) in one pass
@@ -829,6 +872,14 @@ __global__ void __launch_bounds__(256) dcgs_update_df_kernel(int64_t nm, int m, 
 
 // ----------------------------------------------------------------------------
 static inline unsigned nblocks(int64_t n, int th) { return (unsigned)((n + th - 1) / th); }
+
+static void launch_lsq(int m, int restart, const double2* H, const double2* g, const int* kcol, double2* y,
+                       float4* ydf, cudaStream_t st) {
+    const size_t sm = (size_t)restart * sizeof(double2);
+    const bool fits = sm <= 48 * 1024;
+    lsq_kernel<<<m, 32, fits ? sm : 0, st>>>(m, restart, fits ? 1 : 0, H, g, kcol, y, ydf);
+    MWI_CHECK_LAUNCH();
+}
 
 template <typename C>
 void Gmres<C>::reserve(int64_t n_, int m_, int restart_) {
@@ -921,8 +972,8 @@ int Gmres<C>::cycle(const OpFn& A, const OpFn& M, const C* r0, C* x, const doubl
         if (timer) timer(2, ortho);
         else ortho();
         MWI_CUDA(cudaMemsetAsync(nact, 0, sizeof(int), st));
-        arnoldi_kernel<<<nblocks(m, 128), 128, 0, st>>>(m, k, restart, hacc.p, hn2, H.p, cs.p, sn.p, g.p, active,
-                                                        kcol, tol, resid, inv, nact, nullptr);
+        arnoldi_kernel<<<m, 32, 0, st>>>(m, k, restart, hacc.p, hn2, H.p, cs.p, sn.p, g.p, active, kcol, tol, resid,
+                                         inv, nact);
         MWI_CHECK_LAUNCH();
         if (k + 1 < max_steps) {
             scale_kernel<C><<<nblocks(nm, 256), 256, 0, st>>>(n, m, W.p, inv, V.p + (int64_t)(k + 1) * vs);
@@ -932,8 +983,7 @@ int Gmres<C>::cycle(const OpFn& A, const OpFn& M, const C* r0, C* x, const doubl
         MWI_CUDA(cudaStreamSynchronize(st));
         if (n_active_host == 0) { ++k; break; }
     }
-    lsq_kernel<<<nblocks(m, 128), 128, 0, st>>>(m, restart, H.p, g.p, kcol, y.p, nullptr);
-    MWI_CHECK_LAUNCH();
+    launch_lsq(m, restart, H.p, g.p, kcol, y.p, nullptr, st);
     lincomb_kernel<C><<<nblocks(nm, 256), 256, 0, st>>>(n, m, k, Z.p, vs, y.p, x);
     MWI_CHECK_LAUNCH();
     if (resid_host) {
@@ -1015,9 +1065,8 @@ int GmresDF::cycle(const OpA& A, const OpM& M, const float2* r0, float2* x, cons
             dots_reduce_kernel<<<nout, 1024, 0, st>>>(nblk, nout, 0, m, partial.p, h.p, nullptr, nullptr);
             MWI_CHECK_LAUNCH();
             MWI_CUDA(cudaMemsetAsync(nact, 0, sizeof(int), st));
-            arnoldi_dcgs_kernel<<<nblocks(m, 128), 128, 0, st>>>(m, k, restart, last, h.p, H.p, Hp.p, cs.p, sn.p,
-                                                                 g.p, active, kcol, tol, resid, rho, nact, hdf.p,
-                                                                 hdf2.p, scal.p);
+            arnoldi_dcgs_kernel<<<m, 32, 0, st>>>(m, k, restart, last, h.p, H.p, Hp.p, cs.p, sn.p, g.p, active, kcol,
+                                                  tol, resid, rho, nact, hdf.p, hdf2.p, scal.p);
             MWI_CHECK_LAUNCH();
             dcgs_update_df_kernel<<<nblocks(nm, 256), 256, 0, st>>>(nm, m, k, V.p, vs, W.p, hdf.p, hdf2.p, scal.p,
                                                                     last ? 0 : 1);
@@ -1029,8 +1078,7 @@ int GmresDF::cycle(const OpA& A, const OpM& M, const float2* r0, float2* x, cons
         MWI_CUDA(cudaStreamSynchronize(st));
         if (n_active_host == 0) { ++k; break; }
     }
-    lsq_kernel<<<nblocks(m, 128), 128, 0, st>>>(m, restart, H.p, g.p, kcol, y.p, ydf.p);
-    MWI_CHECK_LAUNCH();
+    launch_lsq(m, restart, H.p, g.p, kcol, y.p, ydf.p, st);
     lincomb_df_kernel<<<nblocks(nm, 256), 256, 0, st>>>(nm, m, k, Z.p, nm, ydf.p, x);
     MWI_CHECK_LAUNCH();
     if (iters_used) *iters_used = k;
