@@ -47,8 +47,8 @@ struct CoarseLevel {
     CoarseDev dev;
     std::vector<double2> Aval_h, Ac_h;
     DevBuf<double2> Ac;
-    DevBuf<double2> ws64, inv64, sch64[2];
-    DevBuf<float2> ws32, inv32, sch32[2];
+    DevBuf<double2> ws64, lbuf64, sch64[2];
+    DevBuf<float2> ws32, lbuf32, sch32[2];
     DevBuf<double2> Y64, Z64, upd64, ct64, cq64, q64, w64;
     DevBuf<float2> Y32, Z32, upd32, ct32, cq32, q32, w32;
     DevBuf<int> perturbed;
@@ -56,26 +56,29 @@ struct CoarseLevel {
     double setup_ms = 0;
     size_t bytes() const {
         size_t b = dev.P_rp.bytes() + dev.PT_rp.bytes() + dev.P_col.bytes() + dev.PT_col.bytes() +
-                   dev.P_val.bytes() + dev.PT_val.bytes() + Ac.bytes() + ws64.bytes() + inv64.bytes() +
-                   ws32.bytes() + inv32.bytes() + Y64.bytes() + Z64.bytes() + upd64.bytes() + ct64.bytes() +
+                   dev.P_val.bytes() + dev.PT_val.bytes() + Ac.bytes() + ws64.bytes() + lbuf64.bytes() +
+                   ws32.bytes() + lbuf32.bytes() + Y64.bytes() + Z64.bytes() + upd64.bytes() + ct64.bytes() +
                    cq64.bytes() + q64.bytes() + w64.bytes() + Y32.bytes() + Z32.bytes() + upd32.bytes() +
                    ct32.bytes() + cq32.bytes() + q32.bytes() + w32.bytes() + perturbed.bytes() + ut.tiles.bytes() +
+                   ut.etiles.bytes() +
                    ut.rtiles.bytes();
         for (int k = 0; k < 2; ++k) b += sch64[k].bytes() + sch32[k].bytes();
         return b;
     }
 };
 
-// The factorisation's trailing-update tiles, in its consumption order: per
-// level, per chunk of at most 65535 fronts, per step k of nb pivot columns,
-// the lower-triangle tiles of every front of the chunk with k < p.
+// The factorisation's update tiles, in its consumption order: per level, per
+// chunk of at most 65535 fronts, per step k of nb pivot columns, the tiles of
+// every front of the chunk with k < p.
 void build_update_tiles(const Decomposition& D, int nb, int tile, UpdateTiles& ut, cudaStream_t st) {
-    std::vector<int4> t;
+    std::vector<int4> t, et;
     std::vector<int2> rt;
     ut.nb = nb;
     ut.tile = tile;
     ut.ptr.assign(1, 0);
+    ut.eptr.assign(1, 0);
     ut.rptr.assign(1, 0);
+    auto cover = [tile](int n) { return (n + tile - 1) / tile; };
     for (int l = 0; l < D.n_levels; ++l) {
         const int lo0 = D.level_ptr[l], hi = D.level_ptr[l + 1];
         int pmax = 0;
@@ -87,20 +90,37 @@ void build_update_tiles(const Decomposition& D, int nb, int tile, UpdateTiles& u
                     const int s = D.level_fronts[q];
                     const Front& fr = D.fronts[s];
                     if (k >= fr.p) continue;
-                    const int64_t nrem = (int64_t)fr.p + fr.u - k - std::min(nb, fr.p - k);
-                    const int T = (int)((nrem + tile - 1) / tile);
-                    for (int bi = 0; bi < T; ++bi)
-                        for (int bj = 0; bj <= bi; ++bj) t.push_back(make_int4(s, bi, bj, 0));
-                    for (int r = k + std::min(nb, fr.p - k); r < fr.p + fr.u; r += 128) rt.push_back(make_int2(s, r));
+                    const int f = fr.p + fr.u, r0 = std::min(k + nb, fr.p);
+                    for (int bi = 0; bi < cover(f - r0); ++bi)
+                        for (int bj = 0; bj <= bi && bj < cover(fr.p - r0); ++bj) t.push_back(make_int4(s, bi, bj, 0));
+                    for (int bi = 0; bi < cover(fr.p - r0); ++bi)
+                        for (int bj = 0; bj < cover(r0); ++bj) t.push_back(make_int4(s, bi, bj, 1));
+                    for (int r = r0; r < f; r += 128) rt.push_back(make_int2(s, r));
+                    for (int c = 0; c < k; c += 128) rt.push_back(make_int2(s, -1 - c));
                 }
                 ut.ptr.push_back((int64_t)t.size());
                 ut.rptr.push_back((int64_t)rt.size());
             }
+            // the most pivots first (longest-processing-time order)
+            std::vector<int32_t> order(D.level_fronts.begin() + lo, D.level_fronts.begin() + lo + nf);
+            std::stable_sort(order.begin(), order.end(),
+                             [&](int32_t a, int32_t b) { return D.fronts[a].p > D.fronts[b].p; });
+            for (int32_t s : order) {
+                const Front& fr = D.fronts[s];
+                if (fr.p == 0) continue;
+                for (int bi = 0; bi < cover(fr.u); ++bi) {
+                    for (int bj = 0; bj <= bi; ++bj) et.push_back(make_int4(s, bi, bj, 2));
+                    for (int bj = 0; bj < cover(fr.p); ++bj) et.push_back(make_int4(s, bi, bj, 3));
+                }
+            }
+            ut.eptr.push_back((int64_t)et.size());
         }
     }
     if (t.empty()) t.push_back(make_int4(0, 0, 0, 0));
+    if (et.empty()) et.push_back(make_int4(0, 0, 0, 0));
     if (rt.empty()) rt.push_back(make_int2(0, 0));
     ut.tiles.upload(t, st);
+    ut.etiles.upload(et, st);
     ut.rtiles.upload(rt, st);
     MWI_CUDA(cudaStreamSynchronize(st));
 }
@@ -144,8 +164,8 @@ struct mwi_problem {
     double freq = 0, k0 = 0;
     DevBuf<double2> eps, A_coef, B_coef, Aval, Bval;
     DevBuf<float2> Aval32;
-    DevBuf<double2> ws64, inv64, sch64[2];
-    DevBuf<float2> ws32, inv32, sch32[2];
+    DevBuf<double2> ws64, lbuf64, sch64[2];
+    DevBuf<float2> ws32, lbuf32, sch32[2];
     DevBuf<float> wt;        // tiled, swizzled copy of the c64 panels (tensor-core sweeps)
     DevBuf<int> sweep_err;   // error code of the tensor-core sweeps' bounded waits
     DevBuf<int> sweep_cnt;   // their completion counts (one application at a time: the problem's stream)
@@ -203,7 +223,7 @@ struct mwi_problem {
     // device bytes held by this problem (the mesh and its decomposition are shared)
     size_t device_bytes() const {
         size_t b = eps.bytes() + A_coef.bytes() + B_coef.bytes() + Aval.bytes() + Bval.bytes() + Aval32.bytes() +
-                   ws64.bytes() + inv64.bytes() + ws32.bytes() + inv32.bytes() + perturbed.bytes() + Y64.bytes() +
+                   ws64.bytes() + lbuf64.bytes() + ws32.bytes() + lbuf32.bytes() + perturbed.bytes() + Y64.bytes() +
                    Z64.bytes() + upd64.bytes() + Y32.bytes() + Z32.bytes() + upd32.bytes() + outer.bytes() +
                    inner.bytes() + dfk.bytes() + bgm.bytes() + rc_scratch.bytes() + rc_block.bytes() + Adf.bytes() +
                    Bdf.bytes() + Xdf.bytes() + Rdf.bytes() + U.bytes() + Lam.bytes() + Brhs.bytes() + R.bytes() +
@@ -624,18 +644,18 @@ void upload_fronts(const Decomposition& D, FrontsDev& F, cudaStream_t st) {
         up(F.pdst, pd, st);
     }
     {
-        std::vector<int64_t> io(D.level_fronts.size());
-        F.inv_entries = 0;
+        std::vector<int64_t> lo(nf);
+        F.l_entries = 0;
         for (int l = 0; l < nlev; ++l) {
             int64_t acc = 0;
             for (int q = D.level_ptr[l]; q < D.level_ptr[l + 1]; ++q) {
-                io[q] = acc;
                 const Front& fr = D.fronts[D.level_fronts[q]];
+                lo[D.level_fronts[q]] = acc;
                 acc += (int64_t)fr.p * (fr.p + fr.u);
             }
-            F.inv_entries = std::max(F.inv_entries, acc);
+            F.l_entries = std::max(F.l_entries, acc);
         }
-        up(F.inv_off, io, st);
+        up(F.l_off, lo, st);
     }
     MWI_CUDA(cudaStreamSynchronize(st));
 }
@@ -658,16 +678,16 @@ void coarse_refresh(mwi_problem* P) {
     MWI_CUDA(cudaMemsetAsync(L.perturbed.p, 0, sizeof(int), st));
     if (P->opts.precision != 0) {
         L.ws32.ensure(L.F.ws_total());
-        L.inv32.ensure(std::max<int64_t>(1, L.F.inv_entries));
+        L.lbuf32.ensure(std::max<int64_t>(1, L.F.l_entries));
         for (int k = 0; k < 2; ++k) L.sch32[k].ensure(1);
         float2* sch[2] = {L.sch32[0].p, L.sch32[1].p};
-        factorize_fronts<float2>(L.F, L.ut, L.Ac.p, L.ws32.p, sch, L.inv32.p, L.perturbed.p, st);
+        factorize_fronts<float2>(L.F, L.ut, L.Ac.p, L.ws32.p, sch, L.lbuf32.p, L.perturbed.p, st);
     } else {
         L.ws64.ensure(L.F.ws_total());
-        L.inv64.ensure(std::max<int64_t>(1, L.F.inv_entries));
+        L.lbuf64.ensure(std::max<int64_t>(1, L.F.l_entries));
         for (int k = 0; k < 2; ++k) L.sch64[k].ensure(1);
         double2* sch[2] = {L.sch64[0].p, L.sch64[1].p};
-        factorize_fronts<double2>(L.F, L.ut, L.Ac.p, L.ws64.p, sch, L.inv64.p, L.perturbed.p, st);
+        factorize_fronts<double2>(L.F, L.ut, L.Ac.p, L.ws64.p, sch, L.lbuf64.p, L.perturbed.p, st);
     }
     MWI_CUDA(cudaMemcpyAsync(&L.n_perturbed, L.perturbed.p, sizeof(int), cudaMemcpyDeviceToHost, st));
     MWI_CUDA(cudaStreamSynchronize(st));
@@ -804,14 +824,14 @@ void numeric_setup(mwi_problem* P, bool refactor = true) {
     MWI_CUDA(cudaMemsetAsync(P->perturbed.p, 0, sizeof(int), st));
     if (mixed) {
         P->ws32.ensure(E.F.ws_total());
-        P->inv32.ensure(std::max<int64_t>(1, E.F.inv_entries));
+        P->lbuf32.ensure(std::max<int64_t>(1, E.F.l_entries));
         for (int k = 0; k < 2; ++k) P->sch32[k].ensure(std::max<int64_t>(1, E.F.sch_entries[k]));
         float2* sch[2] = {P->sch32[0].p, P->sch32[1].p};
         std::call_once(E.ut_once[0], [&] {
             build_update_tiles(E.D, factor_block_cols(true), factor_tile_rows(true), E.ut[0], st);
         });
         timed(P, 3, [&] {
-            factorize_fronts<float2>(E.F, E.ut[0], P->Bval.p, P->ws32.p, sch, P->inv32.p, P->perturbed.p, st);
+            factorize_fronts<float2>(E.F, E.ut[0], P->Bval.p, P->ws32.p, sch, P->lbuf32.p, P->perturbed.p, st);
             if (tc_of(P->opts) == 4) {
                 P->wt.ensure(2 * (size_t)E.F.tiled_floats);
                 pack_tiled(E.F.pack_blocks.p, E.F.n_pack_blocks, E.F.f_off.p, E.F.t_off.p, E.F.p.p, E.F.u.p,
@@ -825,14 +845,14 @@ void numeric_setup(mwi_problem* P, bool refactor = true) {
         }
     } else {
         P->ws64.ensure(E.F.ws_total());
-        P->inv64.ensure(std::max<int64_t>(1, E.F.inv_entries));
+        P->lbuf64.ensure(std::max<int64_t>(1, E.F.l_entries));
         for (int k = 0; k < 2; ++k) P->sch64[k].ensure(std::max<int64_t>(1, E.F.sch_entries[k]));
         double2* sch[2] = {P->sch64[0].p, P->sch64[1].p};
         std::call_once(E.ut_once[1], [&] {
             build_update_tiles(E.D, factor_block_cols(false), factor_tile_rows(false), E.ut[1], st);
         });
         timed(P, 3, [&] {
-            factorize_fronts<double2>(E.F, E.ut[1], P->Bval.p, P->ws64.p, sch, P->inv64.p, P->perturbed.p, st);
+            factorize_fronts<double2>(E.F, E.ut[1], P->Bval.p, P->ws64.p, sch, P->lbuf64.p, P->perturbed.p, st);
         });
     }
     MWI_CUDA(cudaMemcpyAsync(&P->n_perturbed, P->perturbed.p, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1864,7 +1884,7 @@ mwi_status mwi_problem_estimate_bytes(mwi_mesh_t M, const mwi_solver_opts* opts,
         double b = nt * 16 + (double)M->A_fu.face.size() * 16 + nnz * 16 + (double)E->D.B_faces.face.size() * 16 +
                    (double)E->B.nnz * 16;
         b += nested ? nnz * 8 : (mixed ? 2 * nnz * 8 : 0);
-        b += ((double)F.ws_total() + (double)F.inv_entries + (double)F.sch_entries[0] + (double)F.sch_entries[1]) * fe;
+        b += ((double)F.ws_total() + (double)F.l_entries + (double)F.sch_entries[0] + (double)F.sch_entries[1]) * fe;
         if (mixed && o.sweep_engine == 4) b += 2.0 * (double)F.tiled_floats * 4 + 4.0 * (double)F.tc_counts();
         // fields of every column (forward, adjoint, right-hand sides), block copies, residual
         b += 3 * n * mall * 16 + 3 * n * m * 16;

@@ -71,6 +71,84 @@ __device__ __forceinline__ dfl df_mul(float ah, float al, float bh, float bl) {
     return r;
 }
 
+// Two FP32 operations per instruction (packed pairs, sm_100 and later), each
+// rounded as the single one is.  They run at the same rate per lane, so they
+// save issue slots, not pipe cycles.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(reinterpret_cast<unsigned long long&>(d))
+        : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)),
+          "l"(reinterpret_cast<const unsigned long long&>(c)));
+    return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;"
+        : "=l"(reinterpret_cast<unsigned long long&>(d))
+        : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
+    return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 d;
+    asm("add.rn.f32x2 %0, %1, %2;"
+        : "=l"(reinterpret_cast<unsigned long long&>(d))
+        : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
+    return d;
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+
+// two double-floats
+struct dfl2 {
+    float2 h, l;
+};
+
+// df_mac1 on both halves, the same operations in the same order: acc += a (bh +
+// bl), nbh = -bh (the product enters as its negative, which the sums subtract)
+__device__ __forceinline__ void df_mac1_2(dfl2& acc, float2 a, float2 bh, float2 nbh, float2 bl) {
+    const float2 np = mul2(a, nbh);
+    float2 e = fma2(a, bh, np);
+    e = fma2(a, bl, e);
+    const float2 s = sub2(acc.h, np);
+    const float2 bb = sub2(s, acc.h);
+    const float2 t = sub2(sub2(acc.h, sub2(s, bb)), add2(np, bb));
+    acc.h = s;
+    acc.l = add2(acc.l, add2(t, e));
+}
+
+// df_mac on both halves: acc += (ah + al) (bh + bl)
+__device__ __forceinline__ void df_mac_2(dfl2& acc, float2 ah, float2 al, float2 bh, float2 nbh, float2 bl) {
+    const float2 np = mul2(ah, nbh);
+    float2 e = fma2(ah, bh, np);
+    e = fma2(ah, bl, e);
+    e = fma2(al, bh, e);
+    const float2 s = sub2(acc.h, np);
+    const float2 bb = sub2(s, acc.h);
+    const float2 t = sub2(sub2(acc.h, sub2(s, bb)), add2(np, bb));
+    acc.h = s;
+    acc.l = add2(acc.l, add2(t, e));
+}
+
+// df_mul on both halves
+__device__ __forceinline__ dfl2 df_mul_2(float2 ah, float2 al, float2 bh, float2 bl) {
+    const float2 p = mul2(ah, bh);
+    float2 e = fma2(ah, bh, make_float2(-p.x, -p.y));
+    e = fma2(ah, bl, e);
+    e = fma2(al, bh, e);
+    dfl2 r;
+    r.h = add2(p, e);
+    r.l = sub2(e, sub2(r.h, p));
+    return r;
+}
+
+__device__ __forceinline__ dfl2 df_norm_2(dfl2 a) {
+    dfl2 r;
+    r.h = add2(a.h, a.l);
+    r.l = sub2(a.l, sub2(r.h, a.h));
+    return r;
+}
+
 // nearest double-float of an FP64 value (FP64 units: use outside hot loops)
 __device__ __forceinline__ float2 df_split(double x) {
     const float h = __double2float_rn(x);

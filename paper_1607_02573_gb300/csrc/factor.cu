@@ -10,21 +10,38 @@
 // The fronts of one assembly-tree depth are processed together, deepest
 // depth first: assemble (entries of B_i, then extend-add of the children's
 // Schur complements), then a blocked right-looking partial factorisation of
-// the p pivot columns (panel kernel + trailing-update kernel) that leaves the
-// Schur complement for the parent.
+// the p pivot columns that leaves the Schur complement for the parent and, in
+// place of the factor, its partitioned inverse for the sweeps.
 // A front (dense, f = p + u, lower triangle used) is stored in two pieces:
-// its p pivot columns as a column-major f x p panel in the factor store (L
-// with unit diagonal implied, D on the diagonal), and its u x u Schur block in
-// a transient buffer shared by the fronts of one level (two buffers, even and
-// odd levels, since a level's blocks are consumed by the next level).  Once a
-// level is factorised, each panel [L11; L21] is replaced by the first p
-// columns of the inverse of [L11 0; L21 I], i.e. [L11^{-1}; -L21 L11^{-1}]
-// (partitioned inverse) with a unit diagonal, and D^{-1} is stored after the
-// panels (indexed by local row), so that each front's part of the ORAS sweeps
-// is one dependency-free dense product per direction (sweep.cu).
+// its p pivot columns as a column-major f x p panel in the factor store, and its
+// u x u Schur block in a transient buffer shared by the fronts of one level (two
+// buffers, even and odd levels, since a level's blocks are consumed by the next
+// level).  The sweeps want the first p columns of the inverse of
+// [L11 0; L21 I], i.e. [L11^{-1}; -L21 L11^{-1}] (partitioned inverse), with a
+// unit diagonal, and D^{-1} after the panels (indexed by local row), so that each
+// front's part of the ORAS sweeps is one dependency-free dense product per
+// direction (sweep.cu).  Of every level, per step of nb pivot columns k ..:
+//   diag    the diagonal block's L D L^T and W, the inverse of its unit lower
+//           triangular factor (replaces the block; D on its diagonal)
+//   rows    L_i = a_i W^T D^{-1} for the rows below (to a scratch panel), and
+//           X_k <- W X_k, X being the inverse's pivot rows left of the step
+//   step    C_ic -= L_i D L_c^T in the remaining pivot columns, and
+//           X_i -= L_i X_k in the remaining pivot rows (Gauss-Jordan, in place
+//           of the factor), as tiles of one launch
+// and after the last step, as tiles of one launch over all p pivots,
+//   end     the Schur block S -= L_2 D L_2^T and the inverse's update rows
+//           X_2 = -L_2 X_1
+// so that a step touches the pivot columns alone, and the larger part of a front
+// is read and written once.  Before, every step updated the whole trailing
+// matrix, and the inverse was formed after the level by column-blocked
+// substitution, eight columns of a front per block, each reading the whole
+// panel.  Whole factorisations, before and now: 3,072 tets 1.34 -> 1.05 ms,
+// 120,288 tets 9.56 -> 8.68 ms, 402,444 tets 39.2 -> 38.0 ms, second order on
+// 53,046 tets 104 -> 82.6 ms, FP64 on 46,080 tets 41.3 -> 38.2 ms.
 #include <algorithm>
 
 #include "common.h"
+#include "df.h"
 #include "kernels.h"
 
 namespace mwi {
@@ -73,101 +90,93 @@ __global__ void extend_add_kernel(const int4* __restrict__ tiles, const int32_t*
     }
 }
 
+constexpr int kUpdateSlab = 8;  // pivots per shared-memory buffer of the products
+
 template <typename C>
 __device__ __forceinline__ bool bad_pivot(C d) {
     typename real_of<C>::type a = d.x * d.x + d.y * d.y;
     return !(a > (typename real_of<C>::type)0) || !isfinite(a);
 }
 
-// Panel step k, part 1: the nb x nb diagonal block of every front of the
-// level, one warp per front (lane r owns row r): LDL^T in shared memory, then
-// M = L^{-T} D^{-1} (upper triangular) by back substitution, lane j taking
-// column j.  The factorised block goes back to the panel (L below the
-// diagonal, D on it) and M's strictly upper part into the block's upper
-// triangle, which the factorisation does not use otherwise (it is cleared when
-// the panel is replaced by its partitioned inverse).
+// Panel step k, diagonal block, one block of NB x 8 threads per front: thread
+// (row lane, column c) holds the entries (row lane + 8 q, c) in registers.  Step
+// j publishes column j (rows below j) and row j (columns left of j), and every
+// thread applies l_r = a_rj / d_j to its rows r > j: right of j the LDL^T update,
+// left of it and in column j the inverse's.  One barrier per step; a warp alone,
+// its lanes over the rows, took 35 us per launch, of which 16 are left.
 template <typename C, int NB>
-__global__ void __launch_bounds__(128) panel_diag_kernel(const int32_t* __restrict__ level_fronts, int lo, int nf,
-                                                         int k, const int32_t* __restrict__ P,
-                                                         const int32_t* __restrict__ U,
-                                                         const int64_t* __restrict__ f_off, C* __restrict__ ws,
-                                                         int* __restrict__ perturbed) {
-    __shared__ C Dgs[4][NB][NB + 1];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int q = blockIdx.x * 4 + warp;
-    if (q >= nf) return;
-    const int s = level_fronts[lo + q];
+__global__ void __launch_bounds__(NB * 8) panel_diag_kernel(const int32_t* __restrict__ level_fronts, int lo, int k,
+                                                            const int32_t* __restrict__ P,
+                                                            const int32_t* __restrict__ U,
+                                                            const int64_t* __restrict__ f_off, C* __restrict__ ws,
+                                                            int* __restrict__ perturbed) {
+    constexpr int Q = NB / 8;
+    __shared__ C colb[2][NB], rowb[2][NB];
+    const int s = level_fronts[lo + blockIdx.x];
     const int p = P[s];
     if (k >= p) return;
     const int64_t f = (int64_t)p + U[s];
     const int nb = min(NB, p - k);
-    C* F = ws + f_off[s];
-    C (*Dg)[NB + 1] = Dgs[warp];
-    {
-        // every load of the lane in flight before the stores
-        C v[NB * NB / 32];
+    C* F = ws + f_off[s] + (int64_t)k * f + k;
+    // rows fastest over the threads: coalesced panel columns
+    const int rl = threadIdx.x & 7, c = threadIdx.x >> 3;
+    C v[Q];
 #pragma unroll
-        for (int t = 0; t < NB * NB / 32; ++t) {
-            const int e = lane + 32 * t, r = e % NB, c = e / NB;
-            v[t] = (r < nb && c < nb && r >= c) ? F[(int64_t)(k + c) * f + k + r] : czero<C>();
-        }
-#pragma unroll
-        for (int t = 0; t < NB * NB / 32; ++t) {
-            const int e = lane + 32 * t;
-            Dg[e % NB][e / NB] = v[t];
-        }
+    for (int q = 0; q < Q; ++q) {
+        const int r = rl + 8 * q;
+        v[q] = (r < nb && c <= r) ? F[(int64_t)c * f + r] : czero<C>();
     }
-    __syncwarp();
-    const int r = lane;
     for (int j = 0; j < nb; ++j) {
-        C d = Dg[j][j];
-        if (bad_pivot(d)) {  // the same value in every lane
-            __syncwarp();
-            if (r == 0) {
-                Dg[j][j] = cmake<C>(1, 0);
+        C* cb = colb[j & 1];
+        C* rb = rowb[j & 1];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int r = rl + 8 * q;
+            if (c == j && r >= j) cb[r] = v[q];
+            if (r == j && c < j) rb[c] = v[q];
+        }
+        __syncthreads();
+        C d = cb[j];
+        if (bad_pivot(d)) {  // the same value in every thread
+            d = cmake<C>(1, 0);
+            if (c == j && rl == (j & 7)) {
+#pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if (q == (j >> 3)) v[q] = d;
                 atomicAdd(perturbed, 1);
             }
-            d = cmake<C>(1, 0);
         }
-        const bool below = r > j && r < nb;
-        C ld = czero<C>();
-        if (below) {
-            const C l = cmul(Dg[r][j], crecip(d));  // l_rj = a_rj / d_j
-            Dg[r][j] = l;
-            ld = cmul(l, d);
-        }
-        __syncwarp();
-        if (below)
-            for (int c = j + 1; c <= r; ++c) Dg[r][c] = csub(Dg[r][c], cmul(ld, Dg[c][j]));
-        __syncwarp();
-    }
-    // column j of M (lane j): y_j = 1, y_r = -sum_{c=r+1..j} L(c, r) y_c for r < j,
-    // kept unscaled in the upper triangle, then scaled by 1 / d_j
-    if (r < nb) {
-        const int j = r;
-        for (int i = j - 1; i >= 0; --i) {
-            C y = cmake<C>(-Dg[j][i].x, -Dg[j][i].y);
-            for (int c = i + 1; c < j; ++c) y = cfms(Dg[c][i], Dg[c][j], y);
-            Dg[i][j] = y;
+        const C rd = crecip(d);
+        const C w = c > j ? cb[c] : (c < j ? rb[c] : czero<C>());
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int r = rl + 8 * q;
+            if (r > j) {
+                const C l = cmul(cb[r], rd);
+                if (c == j) v[q] = cmake<C>(-l.x, -l.y);
+                else if (c <= r) v[q] = cfms(l, w, v[q]);
+            }
         }
     }
-    __syncwarp();
-    for (int e = lane; e < nb * nb; e += 32) {
-        const int rr = e % nb, c = e / nb;
-        C v = Dg[rr][c];
-        if (rr < c) v = cmul(v, crecip(Dg[c][c]));
-        F[(int64_t)(k + c) * f + k + rr] = v;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int r = rl + 8 * q;
+        if (r < nb && c <= r) F[(int64_t)c * f + r] = v[q];
     }
 }
 
-// Panel step k, part 2: the rows below the diagonal block, L_i = a_i M, one
-// thread per row over a tile list (front, first row) of 128-row tiles; M is
-// rebuilt from the block (its strictly upper part, and 1 / D on the diagonal)
+// Panel step k, rows: over a tile list (front, first row) of 128-row tiles below
+// the diagonal block, one thread per row: L_i to the scratch panel; and (front,
+// -1 - first column) of 128-column tiles left of it, one thread per column:
+// X_k <- W X_k.  The products are unrolled over W's triangle; the __syncwarp()s
+// keep its loads from being moved up in a heap that spills the row's registers.
 template <typename C, int NB>
-__global__ void __launch_bounds__(128) panel_rows_kernel(const int2* __restrict__ tiles, int k,
+__global__ void __launch_bounds__(128, 3) panel_rows_kernel(const int2* __restrict__ tiles, int k,
                                                          const int32_t* __restrict__ P, const int32_t* __restrict__ U,
-                                                         const int64_t* __restrict__ f_off, C* __restrict__ ws) {
-    __shared__ C M[NB][NB + 1];
+                                                         const int64_t* __restrict__ f_off,
+                                                         const int64_t* __restrict__ l_off, C* __restrict__ ws,
+                                                         C* __restrict__ lbuf) {
+    __shared__ C W[NB][NB + 1];  // strictly lower: W; diagonal: 1 / D
     const int2 tl = tiles[blockIdx.x];
     const int s = tl.x;
     const int p = P[s];
@@ -180,87 +189,140 @@ __global__ void __launch_bounds__(128) panel_rows_kernel(const int2* __restrict_
 #pragma unroll
         for (int t = 0; t < NB * NB / 128; ++t) {
             const int e = threadIdx.x + 128 * t, r = e % NB, c = e / NB;
-            v[t] = (r < nb && c < nb && r <= c) ? F[(int64_t)(k + c) * f + k + r] : czero<C>();
+            v[t] = (r < nb && c <= r) ? F[(int64_t)(k + c) * f + k + r] : czero<C>();
         }
 #pragma unroll
         for (int t = 0; t < NB * NB / 128; ++t) {
             const int e = threadIdx.x + 128 * t, r = e % NB, c = e / NB;
-            M[r][c] = r == c && r < nb ? crecip(v[t]) : v[t];
+            W[r][c] = r == c && r < nb ? crecip(v[t]) : v[t];
         }
     }
     __syncthreads();
+    if (tl.y < 0) {
+        const int c = -1 - tl.y + threadIdx.x;
+        if (c >= k) return;
+        C* X = F + (int64_t)c * f + k;
+        C x[NB];
+#pragma unroll
+        for (int r = 0; r < NB; ++r) x[r] = r < nb ? X[r] : czero<C>();
+#pragma unroll
+        for (int r = NB - 1; r > 0; --r)
+#pragma unroll
+            for (int q = 0; q < NB; ++q)
+                if (q < r) {
+                    x[r] = cfma(W[r][q], x[q], x[r]);
+                    if (q % 8 == 7) __syncwarp();
+                }
+#pragma unroll
+        for (int r = 0; r < NB; ++r)
+            if (r < nb) X[r] = x[r];
+        return;
+    }
     const int64_t i = (int64_t)tl.y + threadIdx.x;
     if (i >= f) return;
-    // the row's output accumulates in registers while its entries stream in,
+    C* L = lbuf + l_off[s] + (int64_t)k * f + i;
+    // the row's products accumulate in registers while its entries stream in,
     // eight independent loads at a time
     C acc[NB];
 #pragma unroll
     for (int j = 0; j < NB; ++j) acc[j] = czero<C>();
-    for (int c0 = 0; c0 < nb; c0 += 8) {
+#pragma unroll
+    for (int c0 = 0; c0 < NB; c0 += 8) {
         C a[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) a[q] = c0 + q < nb ? F[(int64_t)(k + c0 + q) * f + i] : czero<C>();
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
+        for (int q = 0; q < 8; ++q) {
+            acc[c0 + q] = cadd(acc[c0 + q], a[q]);
 #pragma unroll
-            for (int j = 0; j < NB; ++j) acc[j] = cfma(a[q], M[min(c0 + q, NB - 1)][j], acc[j]);
+            for (int j = 0; j < NB; ++j)
+                if (j > c0 + q) {
+                    acc[j] = cfma(a[q], W[j][c0 + q], acc[j]);
+                    if (j % 8 == 7) __syncwarp();
+                }
+        }
     }
 #pragma unroll
     for (int j = 0; j < NB; ++j)
-        if (j < nb) F[(int64_t)(k + j) * f + i] = acc[j];
+        if (j < nb) L[(int64_t)j * f] = cmul(acc[j], W[j][j]);
 }
 
-// Trailing update of the lower triangle: F[i][c] -= sum_j L[i][j] d_j L[c][j],
-// rows/cols in [k + nb, f).  TILE x TILE output tile per block, 256 threads.
-// One block per tile (front, bi, bj >= ... bi) of the level's tile list for step k.
+// The products of the step (k >= 0, one step's pivots) and of the level's end
+// (k < 0, all pivots), a TILE x TILE output tile per block of 256 threads, over a
+// tile list (front, tile row, tile column, kind):
+//   kStep     rows [r0, f), columns [r0, p), r0 = k + nb: C -= L_i D L_c^T, lower triangle
+//   kStepInv  rows [r0, p), columns [0, r0): X -= L_i X_k; in the step's own
+//             columns X = -L_i W
+//   kSchur    rows and columns [p, f): S -= L_i D L_c^T, lower triangle
+//   kInv      rows [p, f), columns [0, p): X = -L_i X_1
+// Slabs of KS pivots pass through two shared-memory buffers, the next one's loads
+// in flight during the products.  Complex FP32: bound by the FP32 pipe and by
+// how many warps are there to fill it (half busy at 24 warps per SM): four blocks
+// of 64 registers per SM and slabs of 8 take 38.0 ms per factorisation at 402,444
+// tets, slabs of 16 38.8, three blocks of 80 registers 41.0.  A thread's four rows
+// and columns are the pairs 2t, 2t + 1 and 32 + 2t, 32 + 2t + 1, read as 16-byte
+// shared loads; a complex multiply-add is two packed ones, which halves its issue
+// slots (39.8 -> 39.0 ms; with the packed operands laid out in shared memory,
+// twice the shared loads, 41).
+enum { kStep = 0, kStepInv = 1, kSchur = 2, kInv = 3 };
+
 template <typename C, int TILE, int NB>
-__global__ void __launch_bounds__(256, 4) update_kernel(const int4* __restrict__ tiles, int k,
-                                                     const int32_t* __restrict__ P, const int32_t* __restrict__ U,
-                                                     const int64_t* __restrict__ f_off,
-                                                     const int64_t* __restrict__ sch_off, C* __restrict__ ws,
-                                                     C* __restrict__ sch) {
-    const int4 tl = tiles[blockIdx.x];
-    const int s = tl.x, bi = tl.y, bj = tl.z;
-    const int p = P[s];
-    if (k >= p) return;
-    const int64_t f = (int64_t)p + U[s];
-    const int nb = min(NB, p - k);
-    const int64_t r0 = k + nb;
-    const int64_t nrem = f - r0;
-    if ((int64_t)bi * TILE >= nrem) return;
-    C* F = ws + f_off[s];
+__global__ void __launch_bounds__(256, 4)
+    update_kernel(const int4* __restrict__ tiles, int k, const int32_t* __restrict__ P, const int32_t* __restrict__ U,
+                  const int64_t* __restrict__ f_off, const int64_t* __restrict__ sch_off,
+                  const int64_t* __restrict__ l_off, C* __restrict__ ws, const C* __restrict__ lbuf,
+                  C* __restrict__ sch) {
+    constexpr bool kF32 = sizeof(C) == sizeof(float2);
     constexpr int MT = TILE / 16;
-    // complex FP32: a thread's rows (and columns) are the pairs 2t, 2t + 1 and
-    // 32 + 2t, 32 + 2t + 1, read as 16-byte shared loads (rows padded to an even
-    // length so that every pair is 16-byte aligned)
-    constexpr bool kPairs = sizeof(C) == sizeof(float2) && MT == 4;
+    // rows padded to an even length, so that every pair is 16-byte aligned
+    constexpr bool kPairs = kF32 && MT == 4;
     constexpr int LD = kPairs ? TILE + 2 : TILE + 1;
-    __shared__ __align__(16) C As[NB][LD];
-    __shared__ __align__(16) C Bs[NB][LD];
+    constexpr int KS = kUpdateSlab;
+    constexpr int NT = KS * TILE / 256;
+    __shared__ __align__(16) C As[2][KS][LD];
+    __shared__ __align__(16) C Bs[2][KS][LD];
+    const int4 tl = tiles[blockIdx.x];
+    const int s = tl.x, kind = tl.w;
+    const int p = P[s], f = p + U[s];
+    const int r0 = k < 0 ? p : min(k + NB, p);
+    C* const F = ws + f_off[s];
+    const C* const L = lbuf + l_off[s];
     const int tid = threadIdx.x;
-    const int64_t rowA = r0 + (int64_t)bi * TILE, rowB = r0 + (int64_t)bj * TILE;
-    {
-        // every load of the thread in flight before the products and stores
-        constexpr int NT = NB * TILE / 256;
-        C av[NT], bv[NT], dv[NT];
+    const bool inv = (kind & 1) != 0;
+    const int rowA = r0 + tl.y * TILE, endA = kind == kStepInv ? p : f;
+    const int rowB = (inv ? 0 : r0) + tl.z * TILE, endB = kind == kSchur ? f : (kind == kStepInv ? r0 : p);
+    // pivots of the product (X_1 is zero above its diagonal)
+    const int j_end = k < 0 ? p : r0;
+    const int j_beg = k >= 0 ? k : (inv ? rowB / KS * KS : 0);
+    // the inverse's columns: pivots fastest; the factor's: rows fastest
+    auto b_row = [&](int t) { return inv ? (tid + 256 * t) / KS : (tid + 256 * t) % TILE; };
+    auto b_k = [&](int t) { return inv ? (tid + 256 * t) % KS : (tid + 256 * t) / TILE; };
+    C av[NT], bv[NT];
+    auto load = [&](int j0) {
 #pragma unroll
         for (int t = 0; t < NT; ++t) {
-            const int e = tid + 256 * t, ii = e % TILE, j = e / TILE;
-            av[t] = bv[t] = dv[t] = czero<C>();
-            if (j < nb) {
-                dv[t] = F[(int64_t)(k + j) * f + k + j];
-                if (rowA + ii < f) av[t] = F[(int64_t)(k + j) * f + rowA + ii];
-                if (rowB + ii < f) bv[t] = F[(int64_t)(k + j) * f + rowB + ii];
+            const int e = tid + 256 * t, row = rowA + e % TILE, j = j0 + e / TILE;
+            av[t] = bv[t] = czero<C>();
+            if (j < j_end && row < endA) {
+                av[t] = L[(int64_t)j * f + row];
+                if (!inv) av[t] = cmul(av[t], F[(int64_t)j * f + j]);
+            }
+            const int c = rowB + b_row(t), jb = j0 + b_k(t);
+            if (jb < j_end && c < endB) {
+                if (!inv) bv[t] = L[(int64_t)jb * f + c];
+                else if (jb > c) bv[t] = F[(int64_t)c * f + jb];
+                else if (jb == c) bv[t] = cmake<C>(1, 0);
             }
         }
+    };
+    auto store = [&](int buf) {
 #pragma unroll
         for (int t = 0; t < NT; ++t) {
-            const int e = tid + 256 * t, ii = e % TILE, j = e / TILE;
-            As[j][ii] = cmul(av[t], dv[t]);
-            Bs[j][ii] = bv[t];
+            const int e = tid + 256 * t;
+            As[buf][e / TILE][e % TILE] = av[t];
+            Bs[buf][b_k(t)][b_row(t)] = bv[t];
         }
-    }
-    __syncthreads();
+    };
     const int tx = tid % 16, ty = tid / 16;
     // local row of accumulator a (column of b) within the tile
     auto off = [](int t, int a) { return kPairs ? 32 * (a >> 1) + 2 * t + (a & 1) : t + 16 * a; };
@@ -269,210 +331,97 @@ __global__ void __launch_bounds__(256, 4) update_kernel(const int4* __restrict__
     for (int a = 0; a < MT; ++a)
 #pragma unroll
         for (int b = 0; b < MT; ++b) acc[a][b] = czero<C>();
+    load(j_beg);
+    store(0);
+    int buf = 0;
+    for (int j0 = j_beg; j0 < j_end; j0 += KS, buf ^= 1) {
+        __syncthreads();
+        const bool more = j0 + KS < j_end;
+        if (more) load(j0 + KS);
 #pragma unroll 4
-    for (int j = 0; j < NB; ++j) {
-        C av[MT], bv[MT];
-        if constexpr (kPairs) {
+        for (int j = 0; j < KS; ++j) {
+            C a[MT], b[MT];
+            if constexpr (kPairs) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float4 pa = *reinterpret_cast<const float4*>(&As[j][32 * h + 2 * tx]);
-                const float4 pb = *reinterpret_cast<const float4*>(&Bs[j][32 * h + 2 * ty]);
-                av[2 * h] = cmake<C>(pa.x, pa.y);
-                av[2 * h + 1] = cmake<C>(pa.z, pa.w);
-                bv[2 * h] = cmake<C>(pb.x, pb.y);
-                bv[2 * h + 1] = cmake<C>(pb.z, pb.w);
-            }
-        } else {
-#pragma unroll
-            for (int a = 0; a < MT; ++a) av[a] = As[j][tx + 16 * a];
-#pragma unroll
-            for (int b = 0; b < MT; ++b) bv[b] = Bs[j][ty + 16 * b];
-        }
-#pragma unroll
-        for (int a = 0; a < MT; ++a)
-#pragma unroll
-            for (int b = 0; b < MT; ++b) acc[a][b] = cfma(av[a], bv[b], acc[a][b]);
-    }
-    const int u = U[s];
-    C* S = sch + sch_off[s];
-#pragma unroll
-    for (int b = 0; b < MT; ++b) {
-        const int64_t col = rowB + off(ty, b);
-        if (col >= f) continue;
-        // pivot columns live in the panel (ld f), the others in the Schur block (ld u)
-        C* colp = col < p ? F + col * f : S + (col - p) * u - p;
-#pragma unroll
-        for (int a = 0; a < MT; ++a) {
-            const int64_t row = rowA + off(tx, a);
-            if (row < f && row >= col) {
-                C& dst = colp[row];
-                dst = csub(dst, acc[a][b]);
-            }
-        }
-    }
-}
-
-// Partitioned inverse of every front of a level, used by the sweeps.  The
-// panel [L11; L21] is the first p columns of the unit lower triangular
-// [L11 0; L21 I], whose inverse has first p columns [L11^{-1}; -L21 L11^{-1}].
-// Block (front, RC columns c0..) computes those columns for rows >= c0 by
-// column-blocked forward substitution (warp-synchronous 32 x 32 triangles on
-// the pivot rows, row updates below them, the update rows included), writing
-// the strictly lower part to tmp (per front f x p, ld f).
-template <typename C, int RC>
-__global__ void __launch_bounds__(256) invert_panel_kernel(const int32_t* __restrict__ level_fronts, int lo,
-                                                           const int32_t* __restrict__ P,
-                                                           const int32_t* __restrict__ U,
-                                                           const int64_t* __restrict__ f_off,
-                                                           const int64_t* __restrict__ inv_off,
-                                                           const C* __restrict__ ws, C* __restrict__ tmp) {
-    constexpr int RP = RC + 1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* w = reinterpret_cast<C*>(smem_raw);
-    __shared__ C Ld[32][33];
-    const int s = level_fronts[lo + blockIdx.y];
-    const int p = P[s];
-    const int c0 = blockIdx.x * RC;
-    if (c0 >= p) return;
-    const int64_t f = (int64_t)p + U[s];
-    const C* L = ws + f_off[s];
-    C* T = tmp + inv_off[lo + blockIdx.y];
-    const int nr = (int)f - c0;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int e = tid; e < nr * RC; e += 256) {
-        const int i = e / RC, r = e - i * RC;
-        w[i * RP + r] = (i == r) ? cmake<C>(1, 0) : czero<C>();
-    }
-    for (int jb = c0; jb < p; jb += 32) {
-        const int nb = min(32, p - jb);
-        __syncthreads();
-        for (int e = tid; e < 32 * 32; e += 256) {
-            const int i = e & 31, j = e >> 5;
-            Ld[i][j] = (i < nb && j < i) ? L[(int64_t)(jb + j) * f + jb + i] : czero<C>();
-        }
-        __syncthreads();
-        for (int r = warp; r < RC; r += 8) {
-            C val = lane < nb ? w[(jb - c0 + lane) * RP + r] : czero<C>();
-            for (int j = 0; j < nb; ++j) {
-                C x;
-                x.x = __shfl_sync(0xffffffffu, val.x, j);
-                x.y = __shfl_sync(0xffffffffu, val.y, j);
-                val = cfms(Ld[lane][j], x, val);
-            }
-            if (lane < nb) w[(jb - c0 + lane) * RP + r] = val;
-        }
-        __syncthreads();
-        for (int i = jb + nb + tid; i < (int)f; i += 256) {
-            C acc[RC];
-#pragma unroll
-            for (int r = 0; r < RC; ++r) acc[r] = w[(i - c0) * RP + r];
-            // eight panel entries of the row in flight at a time
-            for (int j0 = 0; j0 < nb; j0 += 8) {
-                C l[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) l[q] = j0 + q < nb ? L[(int64_t)(jb + j0 + q) * f + i] : czero<C>();
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const C* wj = w + (jb + min(j0 + q, nb - 1) - c0) * RP;
-#pragma unroll
-                    for (int r = 0; r < RC; ++r) acc[r] = cfms(l[q], wj[r], acc[r]);
+                for (int h = 0; h < 2; ++h) {
+                    const float4 pa = *reinterpret_cast<const float4*>(&As[buf][j][32 * h + 2 * tx]);
+                    const float4 pb = *reinterpret_cast<const float4*>(&Bs[buf][j][32 * h + 2 * ty]);
+                    a[2 * h] = cmake<C>(pa.x, pa.y);
+                    a[2 * h + 1] = cmake<C>(pa.z, pa.w);
+                    b[2 * h] = cmake<C>(pb.x, pb.y);
+                    b[2 * h + 1] = cmake<C>(pb.z, pb.w);
                 }
+            } else {
+#pragma unroll
+                for (int q = 0; q < MT; ++q) a[q] = As[buf][j][off(tx, q)];
+#pragma unroll
+                for (int q = 0; q < MT; ++q) b[q] = Bs[buf][j][off(ty, q)];
             }
 #pragma unroll
-            for (int r = 0; r < RC; ++r) w[(i - c0) * RP + r] = acc[r];
+            for (int x = 0; x < MT; ++x)
+#pragma unroll
+                for (int y = 0; y < MT; ++y) {
+                    if constexpr (kF32) {
+                        acc[x][y] = fma2(both(a[x].x), b[y], acc[x][y]);
+                        acc[x][y] = fma2(both(a[x].y), make_float2(-b[y].y, b[y].x), acc[x][y]);
+                    } else acc[x][y] = cfma(a[x], b[y], acc[x][y]);
+                }
         }
+        if (more) store(buf ^ 1);
     }
-    __syncthreads();
-    for (int e = tid; e < nr * RC; e += 256) {
-        const int i = e / RC, r = e - i * RC;
-        if (c0 + r < p && i > r) T[(int64_t)(c0 + r) * f + c0 + i] = w[i * RP + r];
+    const int u = f - p;
+    C* const Sb = sch + sch_off[s];
+#pragma unroll
+    for (int y = 0; y < MT; ++y) {
+        const int col = rowB + off(ty, y);
+        if (col >= endB) continue;
+        // pivot columns live in the panel (ld f), the others in the Schur block (ld u)
+        C* const colp = col < p ? F + (int64_t)col * f : Sb + (int64_t)(col - p) * u - p;
+        const bool fresh = kind == kInv || (kind == kStepInv && col >= k);  // replaces the factor's entries
+#pragma unroll
+        for (int x = 0; x < MT; ++x) {
+            const int row = rowA + off(tx, x);
+            if (row < endA && row >= col) {
+                C& dst = colp[row];
+                const C v = acc[x][y];
+                dst = fresh ? cmake<C>(-v.x, -v.y) : csub(dst, v);
+            }
+        }
     }
 }
 
-// panel column j <- [L11^{-1}; -L21 L11^{-1}] with a unit diagonal and zeros
-// above it (so that the panel is the sweeps' operand as stored), and
-// 1 / D_jj into dinv at the pivot's local row
+// D^{-1} of every pivot of the level's fronts into dinv at its local row, and the
+// inverse's unit diagonal in D's place
 template <typename C>
-__global__ void copy_inverse_kernel(const int32_t* __restrict__ level_fronts, int lo, const int32_t* __restrict__ P,
-                                    const int32_t* __restrict__ U, const int32_t* __restrict__ start,
-                                    const int32_t* __restrict__ sub, const int64_t* __restrict__ sub_off,
-                                    const int64_t* __restrict__ f_off, const int64_t* __restrict__ inv_off,
-                                    const C* __restrict__ tmp, C* __restrict__ ws, C* __restrict__ dinv) {
-    const int s = level_fronts[lo + blockIdx.y];
+__global__ void finish_diag_kernel(const int32_t* __restrict__ level_fronts, int lo, const int32_t* __restrict__ P,
+                                   const int32_t* __restrict__ U, const int32_t* __restrict__ start,
+                                   const int32_t* __restrict__ sub, const int64_t* __restrict__ sub_off,
+                                   const int64_t* __restrict__ f_off, C* __restrict__ ws, C* __restrict__ dinv) {
+    const int s = level_fronts[lo + blockIdx.x];
     const int p = P[s];
-    const int j = blockIdx.x;
-    if (j >= p) return;
     const int64_t f = (int64_t)p + U[s];
-    C* L = ws + f_off[s] + (int64_t)j * f;
-    const C* T = tmp + inv_off[lo + blockIdx.y] + (int64_t)j * f;
-    const C d = L[j];
-    __syncthreads();
-    // four loads per thread in flight before their stores
-    for (int64_t i0 = 0; i0 < f; i0 += 4 * (int64_t)blockDim.x) {
-        C v[4];
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int64_t i = i0 + t * (int64_t)blockDim.x + threadIdx.x;
-            v[t] = (i < f && i > j) ? T[i] : (i == j ? cmake<C>(1, 0) : czero<C>());
-        }
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int64_t i = i0 + t * (int64_t)blockDim.x + threadIdx.x;
-            if (i < f) L[i] = v[t];
-        }
+    C* F = ws + f_off[s];
+    C* out = dinv + sub_off[sub[s]] + start[s];
+    for (int j = threadIdx.x; j < p; j += blockDim.x) {
+        C& d = F[(int64_t)j * f + j];
+        out[j] = crecip(d);
+        d = cmake<C>(1, 0);
     }
-    if (threadIdx.x == 0) dinv[sub_off[sub[s]] + start[s] + j] = crecip(d);
 }
 
 template <typename C> struct FactorCfg;
 template <> struct FactorCfg<float2> { static constexpr int NB = 32; static constexpr int TILE = 64; };
 template <> struct FactorCfg<double2> { static constexpr int NB = 16; static constexpr int TILE = 32; };
 
-template <typename C, int RC>
-static void invert_level_rc(const FrontsDev& F, int l, int lo, int nf, C* ws, C* tmp, cudaStream_t st) {
-    static bool attr = false;
-    if (!attr) {
-        MWI_CUDA(cudaFuncSetAttribute(invert_panel_kernel<C, RC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      200 * 1024));
-        attr = true;
-    }
-    const int pmax = F.level_pmax[l];
-    const size_t sm = (size_t)F.level_fmax[l] * (RC + 1) * sizeof(C);
-    dim3 grd((pmax + RC - 1) / RC, nf);
-    invert_panel_kernel<C, RC><<<grd, 256, sm, st>>>(F.level_fronts.p, lo, F.p.p, F.u.p, F.f_off.p, F.inv_off.p, ws,
-                                                     tmp);
-    MWI_CHECK_LAUNCH();
-    copy_inverse_kernel<C><<<dim3(pmax, nf), 128, 0, st>>>(F.level_fronts.p, lo, F.p.p, F.u.p, F.start.p, F.sub.p,
-                                                           F.sub_off.p, F.f_off.p, F.inv_off.p, tmp, ws,
-                                                           ws + F.ws_entries);
-    MWI_CHECK_LAUNCH();
-}
-
-// widest column block whose substitution rows fit in 200 KB of shared memory
-template <typename C>
-static void invert_level(const FrontsDev& F, int l, int lo, int nf, C* ws, C* tmp, cudaStream_t st) {
-    const size_t row = (size_t)F.level_fmax[l] * sizeof(C);
-    const size_t lim = 200 * 1024;
-    if constexpr (sizeof(C) == sizeof(float2)) {
-        if (row * 9 <= lim) {
-            invert_level_rc<C, 8>(F, l, lo, nf, ws, tmp, st);
-            return;
-        }
-    }
-    if (row * 5 <= lim) invert_level_rc<C, 4>(F, l, lo, nf, ws, tmp, st);
-    else if (row * 3 <= lim) invert_level_rc<C, 2>(F, l, lo, nf, ws, tmp, st);
-    else if (row * 2 <= lim) invert_level_rc<C, 1>(F, l, lo, nf, ws, tmp, st);
-    else throw Error(MWI_EINVAL, "front too large for the shared-memory inversion");
-}
-
 template <typename C>
 void factorize_fronts(const FrontsDev& F, const UpdateTiles& ut, const double2* Bvals, C* ws, C* const sch[2],
-                      C* inv_tmp, int* perturbed, cudaStream_t st) {
+                      C* lbuf, int* perturbed, cudaStream_t st) {
     constexpr int NB = FactorCfg<C>::NB, TILE = FactorCfg<C>::TILE;
+    static_assert(NB % kUpdateSlab == 0, "a step is whole slabs");
     MWI_REQUIRE(ut.nb == NB && ut.tile == TILE, MWI_EINVAL, "internal: update tiles built for another blocking");
     MWI_CUDA(cudaMemsetAsync(ws, 0, (size_t)(F.ws_entries + F.nloc) * sizeof(C), st));
     const int nlev = (int)F.level_ptr.size() - 1;
-    size_t range = 0, ext = 0;
+    size_t range = 0, ext = 0, end = 0;
     for (int l = 0; l < nlev; ++l) {
         const int lo0 = F.level_ptr[l], hi = F.level_ptr[l + 1];
         C* sch_l = sch[l & 1];
@@ -496,14 +445,14 @@ void factorize_fronts(const FrontsDev& F, const UpdateTiles& ut, const double2* 
             }
             const int pmax = F.level_pmax[l];
             for (int k = 0; k < pmax; k += NB) {
-                panel_diag_kernel<C, NB><<<(nf + 3) / 4, 128, 0, st>>>(F.level_fronts.p, lo, nf, k, F.p.p,
-                                                                       F.u.p, F.f_off.p, ws, perturbed);
+                panel_diag_kernel<C, NB><<<nf, NB * 8, 0, st>>>(F.level_fronts.p, lo, k, F.p.p, F.u.p, F.f_off.p, ws,
+                                                                perturbed);
                 MWI_CHECK_LAUNCH();
                 {
                     const int64_t r0 = ut.rptr[range], r1 = ut.rptr[range + 1];
                     if (r1 > r0) {
-                        panel_rows_kernel<C, NB><<<(unsigned)(r1 - r0), 128, 0, st>>>(ut.rtiles.p + r0, k, F.p.p,
-                                                                                     F.u.p, F.f_off.p, ws);
+                        panel_rows_kernel<C, NB><<<(unsigned)(r1 - r0), 128, 0, st>>>(
+                            ut.rtiles.p + r0, k, F.p.p, F.u.p, F.f_off.p, F.l_off.p, ws, lbuf);
                         MWI_CHECK_LAUNCH();
                     }
                 }
@@ -513,11 +462,23 @@ void factorize_fronts(const FrontsDev& F, const UpdateTiles& ut, const double2* 
                 ++range;
                 if (t1 > t0) {
                     update_kernel<C, TILE, NB><<<(unsigned)(t1 - t0), 256, 0, st>>>(
-                        ut.tiles.p + t0, k, F.p.p, F.u.p, F.f_off.p, F.sch_off.p, ws, sch_l);
+                        ut.tiles.p + t0, k, F.p.p, F.u.p, F.f_off.p, F.sch_off.p, F.l_off.p, ws, lbuf, sch_l);
                     MWI_CHECK_LAUNCH();
                 }
             }
-            invert_level<C>(F, l, lo, nf, ws, inv_tmp, st);
+            {
+                MWI_REQUIRE(end + 1 < ut.eptr.size(), MWI_EINVAL, "internal: update tile list out of step");
+                const int64_t t0 = ut.eptr[end], t1 = ut.eptr[end + 1];
+                ++end;
+                if (t1 > t0) {
+                    update_kernel<C, TILE, NB><<<(unsigned)(t1 - t0), 256, 0, st>>>(
+                        ut.etiles.p + t0, -1, F.p.p, F.u.p, F.f_off.p, F.sch_off.p, F.l_off.p, ws, lbuf, sch_l);
+                    MWI_CHECK_LAUNCH();
+                }
+            }
+            finish_diag_kernel<C><<<nf, 128, 0, st>>>(F.level_fronts.p, lo, F.p.p, F.u.p, F.start.p, F.sub.p,
+                                                      F.sub_off.p, F.f_off.p, ws, ws + F.ws_entries);
+            MWI_CHECK_LAUNCH();
         }
     }
 }

@@ -141,29 +141,31 @@ struct FrontsDev {
     int n_sub = 0;
     TileLists tiles64, tiles32;        // 64-row and 32-row tiles of every level
     std::vector<double> level_pmean, level_fmean;  // host: mean p and f of each level
-    DevBuf<int64_t> inv_off;           // per level position: offset of the front's f x p block
-    int64_t inv_entries = 0;           // largest sum of f p over a level
+    DevBuf<int64_t> l_off;             // per front: offset of its scratch panel (f x p)
+    int64_t l_entries = 0;             // entries of a level's scratch panels, the largest level
 };
 
-// Trailing-update tiles (front, tile row, tile column <= row) of every step
-// of the blocked factorisation, in the order the factorisation consumes them
-// (levels, chunks of 65535 fronts, steps of nb pivot columns); ptr holds the
-// ranges.
+// Tiles (front, tile row, tile column, kind) of the blocked factorisation's
+// products (update_kernel), in the order the factorisation consumes them: of
+// every step (levels, chunks of 65535 fronts, steps of nb pivot columns), and of
+// every level's end (levels, chunks); ptr and eptr hold the ranges.
 struct UpdateTiles {
     int nb = 0, tile = 0;
-    DevBuf<int4> tiles;
-    std::vector<int64_t> ptr;
-    // panel-row tiles (front, first row) of 128 rows below each step's diagonal block
+    DevBuf<int4> tiles, etiles;
+    std::vector<int64_t> ptr, eptr;
+    // panel tiles: (front, first row) of 128 rows below each step's diagonal block,
+    // (front, -1 - first column) of 128 columns left of it
     DevBuf<int2> rtiles;
     std::vector<int64_t> rptr;
 };
 int factor_block_cols(bool fp32);
 int factor_tile_rows(bool fp32);
 
-// ws: factor store (panels); sch[2]: transient Schur buffers (even / odd levels)
+// ws: factor store (panels); sch[2]: transient Schur buffers (even / odd levels);
+// lbuf: scratch panels of a level (FrontsDev::l_entries)
 template <typename C>
 void factorize_fronts(const FrontsDev& F, const UpdateTiles& ut, const double2* Bvals, C* ws, C* const sch[2],
-                      C* inv_tmp, int* perturbed, cudaStream_t st);
+                      C* lbuf, int* perturbed, cudaStream_t st);
 
 // Complex FP32 sweep engine: tc = 0 CUDA cores, 1 mma.sync 3xTF32, 2 mma.sync
 // TF32, 4 tcgen05 TF32 over the tiled panel store wt (cnt: FrontsDev::tc_counts()
