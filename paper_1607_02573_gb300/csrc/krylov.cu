@@ -8,6 +8,7 @@
 // Orthogonalisation is classical Gram-Schmidt applied twice (CGS2): dots of
 // all basis vectors with w in one pass, then one fused update pass.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.h"
 #include "df.h"
@@ -431,6 +432,19 @@ __global__ void __launch_bounds__(256) spmm_df_kernel(int64_t n, const int32_t* 
     for (int c0 = 0; c0 < m; c0 += G) {
         const int c = c0 + lane;
         if (c >= m) break;
+        if constexpr (!RES) {
+            dfl2 acc = {both(0.f), both(0.f)};
+            for (int q = b; q < e; ++q) {
+                const float2 ah = Ah[q], al = Al[q];
+                const float2 xh = Xh[(int64_t)col[q] * m + c];
+                df_mac1_2(acc, xh, both(ah.x), both(-ah.x), both(al.x));
+                df_mac1_2(acc, make_float2(-xh.y, xh.x), both(ah.y), both(-ah.y), both(al.y));
+            }
+            acc = df_norm_2(acc);
+            Wh[row * m + c] = acc.h;
+            Wl[row * m + c] = acc.l;
+            continue;
+        }
         dfl re = {0.f, 0.f}, im = {0.f, 0.f};
         if constexpr (RES) {
             const float2 bh = Bh[row * m + c], bl = Bl[row * m + c];
@@ -440,19 +454,11 @@ __global__ void __launch_bounds__(256) spmm_df_kernel(int64_t n, const int32_t* 
         for (int q = b; q < e; ++q) {
             const float2 ah = Ah[q], al = Al[q];
             const int64_t xi = (int64_t)col[q] * m + c;
-            const float2 xh = Xh[xi];
-            if constexpr (RES) {
-                const float2 xl = Xl[xi];
-                df_mac(re, -ah.x, -al.x, xh.x, xl.x);
-                df_mac(re, ah.y, al.y, xh.y, xl.y);
-                df_mac(im, -ah.x, -al.x, xh.y, xl.y);
-                df_mac(im, -ah.y, -al.y, xh.x, xl.x);
-            } else {
-                df_mac1(re, xh.x, ah.x, al.x);
-                df_mac1(re, -xh.y, ah.y, al.y);
-                df_mac1(im, xh.y, ah.x, al.x);
-                df_mac1(im, xh.x, ah.y, al.y);
-            }
+            const float2 xh = Xh[xi], xl = Xl[xi];
+            df_mac(re, -ah.x, -al.x, xh.x, xl.x);
+            df_mac(re, ah.y, al.y, xh.y, xl.y);
+            df_mac(im, -ah.x, -al.x, xh.y, xl.y);
+            df_mac(im, -ah.y, -al.y, xh.x, xl.x);
         }
         re = df_norm(re);
         im = df_norm(im);
@@ -461,25 +467,48 @@ __global__ void __launch_bounds__(256) spmm_df_kernel(int64_t n, const int32_t* 
     }
 }
 
-// The same product for an even m >= 32 with two adjacent columns per lane (16
-// lanes per row, 16-byte loads of the right-hand sides): four independent
-// accumulation chains per thread instead of two.  Entries are applied in the
-// same ascending order, so the results are the same bit for bit.
-template <bool RES>
+// The same product for an even m with two adjacent columns per lane (16-byte
+// loads of the right-hand sides; G lanes per row, the power of two at or above
+// m / 2, at most 16): four independent accumulation chains per thread instead of
+// two.  Entries are applied in the same ascending order, so the results are the
+// same bit for bit.
+// w = A z (RES = false): the error-free products and sums bound it; they run on
+// (re, im) pairs, two operations per instruction.  458,220 rows, 7.35 M entries,
+// ms per product: 32 columns 0.48 -> 0.45, 31 columns (one per lane, 32 lanes a
+// row instead of four passes of 8) 0.57 -> 0.46, 6 columns 0.156 -> 0.126.
+template <int G, bool RES>
 __global__ void __launch_bounds__(256) spmm_df2_kernel(int64_t n, const int32_t* __restrict__ rp,
                                                        const int32_t* __restrict__ col, const float2* __restrict__ Ah,
                                                        const float2* __restrict__ Al, const float4* __restrict__ Xh,
                                                        const float4* __restrict__ Xl, const float4* __restrict__ Bh,
                                                        const float4* __restrict__ Bl, float4* __restrict__ Wh,
                                                        float4* __restrict__ Wl, int m) {
-    const int lane = threadIdx.x & 15;
-    const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 4;
+    const int lane = threadIdx.x % G;
+    const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
     if (row >= n) return;
     const int h = m >> 1;  // column pairs per row
     const int b = rp[row], e = rp[row + 1];
-    for (int c0 = 0; c0 < h; c0 += 16) {
+    for (int c0 = 0; c0 < h; c0 += G) {
         const int c = c0 + lane;
         if (c >= h) break;
+        if constexpr (!RES) {
+            dfl2 a0 = {both(0.f), both(0.f)}, a1 = a0;
+            for (int q = b; q < e; ++q) {
+                const float2 ah = Ah[q], al = Al[q];
+                const float4 xh = Xh[(int64_t)col[q] * h + c];
+                const float2 rh = both(ah.x), nrh = both(-ah.x), rl = both(al.x);
+                const float2 ih = both(ah.y), nih = both(-ah.y), il = both(al.y);
+                df_mac1_2(a0, make_float2(xh.x, xh.y), rh, nrh, rl);
+                df_mac1_2(a1, make_float2(xh.z, xh.w), rh, nrh, rl);
+                df_mac1_2(a0, make_float2(-xh.y, xh.x), ih, nih, il);
+                df_mac1_2(a1, make_float2(-xh.w, xh.z), ih, nih, il);
+            }
+            a0 = df_norm_2(a0);
+            a1 = df_norm_2(a1);
+            Wh[row * h + c] = make_float4(a0.h.x, a0.h.y, a1.h.x, a1.h.y);
+            Wl[row * h + c] = make_float4(a0.l.x, a0.l.y, a1.l.x, a1.l.y);
+            continue;
+        }
         dfl re0 = {0.f, 0.f}, im0 = {0.f, 0.f}, re1 = {0.f, 0.f}, im1 = {0.f, 0.f};
         if constexpr (RES) {
             const float4 bh = Bh[row * h + c], bl = Bl[row * h + c];
@@ -491,27 +520,15 @@ __global__ void __launch_bounds__(256) spmm_df2_kernel(int64_t n, const int32_t*
         for (int q = b; q < e; ++q) {
             const float2 ah = Ah[q], al = Al[q];
             const int64_t xi = (int64_t)col[q] * h + c;
-            const float4 xh = Xh[xi];
-            if constexpr (RES) {
-                const float4 xl = Xl[xi];
-                df_mac(re0, -ah.x, -al.x, xh.x, xl.x);
-                df_mac(re0, ah.y, al.y, xh.y, xl.y);
-                df_mac(im0, -ah.x, -al.x, xh.y, xl.y);
-                df_mac(im0, -ah.y, -al.y, xh.x, xl.x);
-                df_mac(re1, -ah.x, -al.x, xh.z, xl.z);
-                df_mac(re1, ah.y, al.y, xh.w, xl.w);
-                df_mac(im1, -ah.x, -al.x, xh.w, xl.w);
-                df_mac(im1, -ah.y, -al.y, xh.z, xl.z);
-            } else {
-                df_mac1(re0, xh.x, ah.x, al.x);
-                df_mac1(re0, -xh.y, ah.y, al.y);
-                df_mac1(im0, xh.y, ah.x, al.x);
-                df_mac1(im0, xh.x, ah.y, al.y);
-                df_mac1(re1, xh.z, ah.x, al.x);
-                df_mac1(re1, -xh.w, ah.y, al.y);
-                df_mac1(im1, xh.w, ah.x, al.x);
-                df_mac1(im1, xh.z, ah.y, al.y);
-            }
+            const float4 xh = Xh[xi], xl = Xl[xi];
+            df_mac(re0, -ah.x, -al.x, xh.x, xl.x);
+            df_mac(re0, ah.y, al.y, xh.y, xl.y);
+            df_mac(im0, -ah.x, -al.x, xh.y, xl.y);
+            df_mac(im0, -ah.y, -al.y, xh.x, xl.x);
+            df_mac(re1, -ah.x, -al.x, xh.z, xl.z);
+            df_mac(re1, ah.y, al.y, xh.w, xl.w);
+            df_mac(im1, -ah.x, -al.x, xh.w, xl.w);
+            df_mac(im1, -ah.y, -al.y, xh.z, xl.z);
         }
         re0 = df_norm(re0);
         im0 = df_norm(im0);
@@ -814,60 +831,104 @@ __global__ void __launch_bounds__(256) dcgs_update_df_kernel(int64_t nm, int m, 
     const int c = (int)(e % m);
     const float4 s1 = scal[c], s2 = scal[m + c];
     float2* vk = V + (int64_t)k * vstride;
-    const float2 vh = vk[e], vl = vk[nm + e], wh = W[e], wl = W[nm + e];
-    // q accumulator: v_k / nu; w accumulator: w / rho_k + v_k (-c_k / (nu rho_k))
-    dfl qr = df_mul(vh.x, vl.x, s1.x, s1.y), qi = df_mul(vh.y, vl.y, s1.x, s1.y);
-    dfl wr = df_mul(wh.x, wl.x, s1.z, s1.w), wi = df_mul(wh.y, wl.y, s1.z, s1.w);
-    df_mac(wr, vh.x, vl.x, s2.x, s2.y);
-    df_mac(wr, -vh.y, -vl.y, s2.z, s2.w);
-    df_mac(wi, vh.x, vl.x, s2.z, s2.w);
-    df_mac(wi, vh.y, vl.y, s2.x, s2.y);
-    int i = 0;
-    for (; i + 2 <= k; i += 2) {
-        float2 qh[2], ql[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            qh[u] = V[(int64_t)(i + u) * vstride + e];
-            ql[u] = V[(int64_t)(i + u) * vstride + nm + e];
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const float4 a = coefQ[(i + u) * m + c], b = coefW[(i + u) * m + c];
-            df_mac(qr, qh[u].x, ql[u].x, a.x, a.y);
-            df_mac(qr, -qh[u].y, -ql[u].y, a.z, a.w);
-            df_mac(qi, qh[u].x, ql[u].x, a.z, a.w);
-            df_mac(qi, qh[u].y, ql[u].y, a.x, a.y);
-            df_mac(wr, qh[u].x, ql[u].x, b.x, b.y);
-            df_mac(wr, -qh[u].y, -ql[u].y, b.z, b.w);
-            df_mac(wi, qh[u].x, ql[u].x, b.z, b.w);
-            df_mac(wi, qh[u].y, ql[u].y, b.x, b.y);
-        }
-    }
-    for (; i < k; ++i) {
-        const float2 qh = V[(int64_t)i * vstride + e], ql = V[(int64_t)i * vstride + nm + e];
+    const float2 vh = vk[e], vl = vk[nm + e];
+    // q accumulator: v_k / nu; x accumulator: w / rho_k + v_k (-c_k / (nu rho_k));
+    // (re, im) pairs, the operations in the order of the even-m form
+    dfl2 q = df_mul_2(vh, vl, both(s1.x), both(s1.y)), x = df_mul_2(W[e], W[nm + e], both(s1.z), both(s1.w));
+    df_mac_2(x, vh, vl, both(s2.x), both(-s2.x), both(s2.y));
+    df_mac_2(x, make_float2(-vh.y, vh.x), make_float2(-vl.y, vl.x), both(s2.z), both(-s2.z), both(s2.w));
+#pragma unroll 2
+    for (int i = 0; i < k; ++i) {
+        const float2 uh = V[(int64_t)i * vstride + e], ul = V[(int64_t)i * vstride + nm + e];
+        const float2 th = make_float2(-uh.y, uh.x), tl = make_float2(-ul.y, ul.x);
         const float4 a = coefQ[i * m + c], b = coefW[i * m + c];
-        df_mac(qr, qh.x, ql.x, a.x, a.y);
-        df_mac(qr, -qh.y, -ql.y, a.z, a.w);
-        df_mac(qi, qh.x, ql.x, a.z, a.w);
-        df_mac(qi, qh.y, ql.y, a.x, a.y);
-        df_mac(wr, qh.x, ql.x, b.x, b.y);
-        df_mac(wr, -qh.y, -ql.y, b.z, b.w);
-        df_mac(wi, qh.x, ql.x, b.z, b.w);
-        df_mac(wi, qh.y, ql.y, b.x, b.y);
+        df_mac_2(q, uh, ul, both(a.x), both(-a.x), both(a.y));
+        df_mac_2(q, th, tl, both(a.z), both(-a.z), both(a.w));
+        df_mac_2(x, uh, ul, both(b.x), both(-b.x), both(b.y));
+        df_mac_2(x, th, tl, both(b.z), both(-b.z), both(b.w));
     }
     if (k > 0) {
-        qr = df_norm(qr);
-        qi = df_norm(qi);
-        vk[e] = make_float2(qr.h, qi.h);
-        vk[nm + e] = make_float2(qr.l, qi.l);
+        q = df_norm_2(q);
+        vk[e] = q.h;
+        vk[nm + e] = q.l;
     }
     if (write_next) {
-        wr = df_norm(wr);
-        wi = df_norm(wi);
+        x = df_norm_2(x);
         float2* vn = V + (int64_t)(k + 1) * vstride;
-        vn[e] = make_float2(wr.h, wi.h);
-        vn[nm + e] = make_float2(wr.l, wi.l);
+        vn[e] = x.h;
+        vn[nm + e] = x.l;
     }
+}
+
+// The same pass for an even m, bound by memory (16 k + 64 bytes per element): a
+// thread takes two adjacent columns (16-byte accesses) of two rows, so that the
+// coefficients and their packed forms serve both, and has the next basis vector
+// on its way while it works on one.  A block is (column pairs) x (rows), rows
+// contiguous in memory.  With one column of one row per thread the Arnoldi steps
+// of a solve (458,220 rows, 32 columns, 24 steps, dot products included) took
+// 25.8 ms, now 24.0.
+__global__ void __launch_bounds__(256) dcgs_update_df2_kernel(int64_t n, int h, int k, float4* __restrict__ V,
+                                                              int64_t vstride, const float4* __restrict__ W,
+                                                              const float4* __restrict__ coefQ,
+                                                              const float4* __restrict__ coefW,
+                                                              const float4* __restrict__ scal, int write_next) {
+    const int cp = blockIdx.y * blockDim.x + threadIdx.x;
+    if (cp >= h) return;
+    const int64_t r0 = blockIdx.x * (int64_t)(2 * blockDim.y) + threadIdx.y;
+    if (r0 >= n) return;
+    const int64_t nh = n * h;
+    const bool two = r0 + blockDim.y < n;
+    const int64_t e0 = r0 * h + cp, e1 = two ? e0 + (int64_t)blockDim.y * h : e0;
+    const int m = 2 * h;
+    float4* const vk = V + (int64_t)k * vstride;
+    struct Pair { float4 h[2], l[2]; };  // two columns of the two rows
+    auto load = [&](const float4* p) { return Pair{{p[e0], p[e1]}, {p[nh + e0], p[nh + e1]}}; };
+    auto lo2 = [](float4 v, int c) { return c ? make_float2(v.z, v.w) : make_float2(v.x, v.y); };
+    const Pair v = load(vk), w = load(W);
+    Pair next = k > 0 ? load(V) : v;
+    dfl2 q[2][2], x[2][2];  // [column][row]: q_k and v_{k+1}
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const float4 s1 = scal[2 * cp + c], s2 = scal[m + 2 * cp + c];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const float2 vh = lo2(v.h[r], c), vl = lo2(v.l[r], c);
+            q[c][r] = df_mul_2(vh, vl, both(s1.x), both(s1.y));
+            x[c][r] = df_mul_2(lo2(w.h[r], c), lo2(w.l[r], c), both(s1.z), both(s1.w));
+            df_mac_2(x[c][r], vh, vl, both(s2.x), both(-s2.x), both(s2.y));
+            df_mac_2(x[c][r], make_float2(-vh.y, vh.x), make_float2(-vl.y, vl.x), both(s2.z), both(-s2.z),
+                     both(s2.w));
+        }
+    }
+    for (int i = 0; i < k; ++i) {
+        const Pair u = next;
+        if (i + 1 < k) next = load(V + (int64_t)(i + 1) * vstride);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const float4 a = coefQ[i * m + 2 * cp + c], b = coefW[i * m + 2 * cp + c];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const float2 uh = lo2(u.h[r], c), ul = lo2(u.l[r], c);
+                const float2 th = make_float2(-uh.y, uh.x), tl = make_float2(-ul.y, ul.x);
+                df_mac_2(q[c][r], uh, ul, both(a.x), both(-a.x), both(a.y));
+                df_mac_2(q[c][r], th, tl, both(a.z), both(-a.z), both(a.w));
+                df_mac_2(x[c][r], uh, ul, both(b.x), both(-b.x), both(b.y));
+                df_mac_2(x[c][r], th, tl, both(b.z), both(-b.z), both(b.w));
+            }
+        }
+    }
+    auto put = [&](float4* p, dfl2 (&a)[2][2]) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            if (r == 1 && !two) continue;
+            const int64_t e = r ? e1 : e0;
+            const dfl2 c0 = df_norm_2(a[0][r]), c1 = df_norm_2(a[1][r]);
+            p[e] = make_float4(c0.h.x, c0.h.y, c1.h.x, c1.h.y);
+            p[nh + e] = make_float4(c0.l.x, c0.l.y, c1.l.x, c1.l.y);
+        }
+    };
+    if (k > 0) put(vk, q);
+    if (write_next) put(vk + vstride, x);
 }
 
 // ----------------------------------------------------------------------------
@@ -1068,8 +1129,15 @@ int GmresDF::cycle(const OpA& A, const OpM& M, const float2* r0, float2* x, cons
             arnoldi_dcgs_kernel<<<m, 32, 0, st>>>(m, k, restart, last, h.p, H.p, Hp.p, cs.p, sn.p, g.p, active, kcol,
                                                   tol, resid, rho, nact, hdf.p, hdf2.p, scal.p);
             MWI_CHECK_LAUNCH();
-            dcgs_update_df_kernel<<<nblocks(nm, 256), 256, 0, st>>>(nm, m, k, V.p, vs, W.p, hdf.p, hdf2.p, scal.p,
-                                                                    last ? 0 : 1);
+            if (m % 2 == 0) {
+                const int h = m / 2, hx = std::min(h, 256), hy = 256 / hx;
+                dcgs_update_df2_kernel<<<dim3(nblocks(n, 2 * hy), (h + hx - 1) / hx), dim3(hx, hy), 0, st>>>(
+                    n, h, k, reinterpret_cast<float4*>(V.p), vs / 2, reinterpret_cast<const float4*>(W.p), hdf.p,
+                    hdf2.p, scal.p, last ? 0 : 1);
+            } else {
+                dcgs_update_df_kernel<<<nblocks(nm, 256), 256, 0, st>>>(nm, m, k, V.p, vs, W.p, hdf.p, hdf2.p,
+                                                                        scal.p, last ? 0 : 1);
+            }
             MWI_CHECK_LAUNCH();
         };
         if (timer) timer(2, ortho);
@@ -1085,55 +1153,45 @@ int GmresDF::cycle(const OpA& A, const OpM& M, const float2* r0, float2* x, cons
     return k;
 }
 
-void spmm_df(int64_t n, const int32_t* row_ptr, const int32_t* col, const float2* A, int64_t nnz, const float2* x,
-             float2* w, int m, cudaStream_t st) {
+template <bool RES>
+static void launch_spmm_df(int64_t n, const int32_t* row_ptr, const int32_t* col, const float2* A, int64_t nnz,
+                           const float2* x, const float2* b, float2* w, int m, cudaStream_t st) {
     const int th = 256;
     const int64_t nm = n * m;
-    if (m >= 32 && (m & 1) == 0) {
-        spmm_df2_kernel<false><<<(unsigned)((n * 16 + th - 1) / th), th, 0, st>>>(
-            n, row_ptr, col, A, A + nnz, reinterpret_cast<const float4*>(x), nullptr, nullptr, nullptr,
-            reinterpret_cast<float4*>(w), reinterpret_cast<float4*>(w + nm), m);
-        MWI_CHECK_LAUNCH();
-        return;
+    auto f4 = [](const float2* p) { return reinterpret_cast<const float4*>(p); };
+    auto pairs = [&](auto g) {
+        constexpr int G = decltype(g)::value;
+        spmm_df2_kernel<G, RES><<<(unsigned)((n * G + th - 1) / th), th, 0, st>>>(
+            n, row_ptr, col, A, A + nnz, f4(x), RES ? f4(x + nm) : nullptr, RES ? f4(b) : nullptr,
+            RES ? f4(b + nm) : nullptr, reinterpret_cast<float4*>(w), reinterpret_cast<float4*>(w + nm), m);
+    };
+    auto singles = [&](auto g) {
+        constexpr int G = decltype(g)::value;
+        spmm_df_kernel<G, RES><<<(unsigned)((n * G + th - 1) / th), th, 0, st>>>(
+            n, row_ptr, col, A, A + nnz, x, RES ? x + nm : nullptr, b, RES ? b + nm : nullptr, w, w + nm, m);
+    };
+    if ((m & 1) == 0) {
+        if (m > 16) pairs(std::integral_constant<int, 16>());
+        else if (m > 8) pairs(std::integral_constant<int, 8>());
+        else if (m > 4) pairs(std::integral_constant<int, 4>());
+        else pairs(std::integral_constant<int, 2>());
+    } else {
+        if (m > 16) singles(std::integral_constant<int, 32>());
+        else if (m > 8) singles(std::integral_constant<int, 16>());
+        else if (m > 4) singles(std::integral_constant<int, 8>());
+        else singles(std::integral_constant<int, 4>());
     }
-    const int G = m >= 32 ? 32 : (m >= 8 ? 8 : 4);
-    const unsigned blocks = (unsigned)((n * G + th - 1) / th);
-    if (G == 32)
-        spmm_df_kernel<32, false><<<blocks, th, 0, st>>>(n, row_ptr, col, A, A + nnz, x, nullptr, nullptr, nullptr, w,
-                                                         w + nm, m);
-    else if (G == 8)
-        spmm_df_kernel<8, false><<<blocks, th, 0, st>>>(n, row_ptr, col, A, A + nnz, x, nullptr, nullptr, nullptr, w,
-                                                        w + nm, m);
-    else
-        spmm_df_kernel<4, false><<<blocks, th, 0, st>>>(n, row_ptr, col, A, A + nnz, x, nullptr, nullptr, nullptr, w,
-                                                        w + nm, m);
     MWI_CHECK_LAUNCH();
+}
+
+void spmm_df(int64_t n, const int32_t* row_ptr, const int32_t* col, const float2* A, int64_t nnz, const float2* x,
+             float2* w, int m, cudaStream_t st) {
+    launch_spmm_df<false>(n, row_ptr, col, A, nnz, x, nullptr, w, m, st);
 }
 
 void residual_df(int64_t n, const int32_t* row_ptr, const int32_t* col, const float2* A, int64_t nnz, const float2* b,
                  const float2* x, float2* r, int m, cudaStream_t st) {
-    const int th = 256;
-    const int64_t nm = n * m;
-    if (m >= 32 && (m & 1) == 0) {
-        spmm_df2_kernel<true><<<(unsigned)((n * 16 + th - 1) / th), th, 0, st>>>(
-            n, row_ptr, col, A, A + nnz, reinterpret_cast<const float4*>(x), reinterpret_cast<const float4*>(x + nm),
-            reinterpret_cast<const float4*>(b), reinterpret_cast<const float4*>(b + nm), reinterpret_cast<float4*>(r),
-            reinterpret_cast<float4*>(r + nm), m);
-        MWI_CHECK_LAUNCH();
-        return;
-    }
-    const int G = m >= 32 ? 32 : (m >= 8 ? 8 : 4);
-    const unsigned blocks = (unsigned)((n * G + th - 1) / th);
-    if (G == 32)
-        spmm_df_kernel<32, true><<<blocks, th, 0, st>>>(n, row_ptr, col, A, A + nnz, x, x + nm, b, b + nm, r, r + nm,
-                                                        m);
-    else if (G == 8)
-        spmm_df_kernel<8, true><<<blocks, th, 0, st>>>(n, row_ptr, col, A, A + nnz, x, x + nm, b, b + nm, r, r + nm,
-                                                       m);
-    else
-        spmm_df_kernel<4, true><<<blocks, th, 0, st>>>(n, row_ptr, col, A, A + nnz, x, x + nm, b, b + nm, r, r + nm,
-                                                       m);
-    MWI_CHECK_LAUNCH();
+    launch_spmm_df<true>(n, row_ptr, col, A, nnz, x, b, r, m, st);
 }
 
 void split_c128(int64_t count, const double2* a, float2* out, cudaStream_t st) {
