@@ -54,7 +54,9 @@
 // Why one launch: with a launch per level and direction (and one more for the
 // extend-add of the pivot rows) every level ended in a partly filled last wave
 // and began with the set-up of all CTAs; subdomains, whose levels are
-// independent of each other, now overlap across levels.  Measured: XX3.
+// independent of each other, now overlap across levels.  Per application of 32
+// columns on 402,444 tets, gather and scatter included: 1.83 -> 1.42 ms; of one
+// column on 7,392 tets 160 -> 70 us.
 // Warp roles:
 //   warp 0      streams the panel blocks by bulk copies, which depend on no
 //               other tile
@@ -64,14 +66,14 @@
 //               rows into the B operand by 16-byte asynchronous copies (16 lanes
 //               a row).  The chain of a stage -- free, gathered, multiplied --
 //               sets its rate: with a K-major B, which took a transposition
-//               through shared memory between the two, the same launch ran
-//               XX4, with one bulk copy per run of contiguous rows XX5.
+//               through shared memory between the two, an application took
+//               2.10 ms where this one took 1.82 (conversions to FP64 included)
 //   warps 4-7   epilogue: tcgen05.ld, complex combine, D^{-1} scaling or
 //               extend-add, global stores, the front's count
 //   warp 8      draws the tiles, one ahead of warp 0 (a long tile does not hold
 //               back one that others wait for): descriptor into the ring,
-//               update-row indices into shared memory, the first part of the
-//               panel into L2
+//               update-row indices into shared memory.  (Fetching the first part
+//               of the tile's panel into L2 as well cost 1.75 against 1.55 ms.)
 // Stages (per CTA, two CTAs per SM) form a ring shared by all tiles of the CTA,
 // so loads of the next tile overlap the products and the epilogue of the
 // current one.  The rows are copied in units of 16 bytes, so the engine needs an
@@ -108,7 +110,6 @@ constexpr int kSmemBytes =
 static_assert(kSmemBytes * kCtasPerSm <= 228 * 1024 - 2048, "shared memory per SM");
 constexpr long long kWaitLimit = 1ll << 24;
 constexpr int kDepLimit = 1 << 22;          // polls of a dependency count (a few seconds)
-constexpr int kAheadSteps = 32;             // K steps of the next tile's panel fetched into L2
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -205,9 +206,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-__device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
 // 16 bytes global -> shared past L1, asynchronously (bytes = 0: zeros, nothing
 // is read); copies_arrive: this thread's arrival on the barrier once its copies
 // so far have landed
@@ -216,6 +214,18 @@ __device__ __forceinline__ void copy16(uint32_t dst, const void* src, uint32_t b
 }
 __device__ __forceinline__ void copies_arrive(uint32_t bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+// 32 bytes per access (sm_100 and later), 32-byte aligned; loads past L1
+__device__ __forceinline__ void store32(float2* p, const float* v) {
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
+__device__ __forceinline__ void load32(const float2* p, float* v) {
+    asm volatile("ld.global.cg.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p)
+                 : "memory");
 }
 __device__ __forceinline__ int ld_acquire(const int* p) {
     int v;
@@ -519,9 +529,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                 bulk_g2s(smem_u32(sur + (nsur % kSurBufs) * kUrCache), urows + (slot->d.u_off - off), bytes, bar);
             }
             nsur += indices_cached(G) ? 1 : 0;
-            if (lane < min(G.nk, kAheadSteps))
-                l2_prefetch(wt + slot->d.a_off + ((int64_t)(G.k0 + lane) * G.cstride + G.g0) * 128,
-                            (uint32_t)G.ng * 512u);
         }
         if (!ok && lane == 0)
             for (int q = max(0, nsur - kSurBufs); q < nsur; ++q)
@@ -564,6 +571,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             if (!(ok = mbar_wait(tfull_bar(buf), (it >> 1) & 1, abort_flag, err, 5))) break;
             tc_fence_after();
             const uint32_t t0 = tmem + ((uint32_t)(lg * 32) << 16) + buf * 128;
+            // whole 32-byte accesses: a lane's row is a line of its own, so an access
+            // of the warp takes 32 passes whatever its width (32 columns, 402,444 tets:
+            // 1.82 -> 1.75 ms; 64 columns 2.93 -> 2.72 ms)
+            const bool wide = nc == 32 && (m & 3) == 0;
             // two halves of 16 complex columns: tensor-memory loads, combine,
             // D^{-1} or the rows to add, stores; the accumulator is released
             // once the second half is in registers.  Rows that other tiles of
@@ -604,6 +615,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                                                     ? upd + (int64_t)(k ? src.y : src.x) * m + c0 + cb
                                                     : nullptr);
                     if (!a) continue;
+                    if (wide) {
+                        float v[32];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) load32(a + 4 * q, v + 8 * q);
+#pragma unroll
+                        for (int q = 0; q < 32; ++q) o[q] += v[q];
+                        continue;
+                    }
 #pragma unroll
                     for (int q = 0; q < 8; ++q)
                         if (cb + 2 * q < nc) {
@@ -613,6 +632,11 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                             o[4 * q + 2] += v.z;
                             o[4 * q + 3] += v.w;
                         }
+                }
+                if (wide) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) store32(dst + cb + 4 * q, o + 8 * q);
+                    continue;
                 }
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
