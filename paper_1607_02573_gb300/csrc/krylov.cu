@@ -8,6 +8,7 @@
 // Orthogonalisation is classical Gram-Schmidt applied twice (CGS2): dots of
 // all basis vectors with w in one pass, then one fused update pass.
 #include <algorithm>
+#include <mutex>
 #include <type_traits>
 
 #include "common.h"
@@ -493,16 +494,22 @@ __global__ void __launch_bounds__(256) spmm_df2_kernel(int64_t n, const int32_t*
         if (c >= h) break;
         if constexpr (!RES) {
             dfl2 a0 = {both(0.f), both(0.f)}, a1 = a0;
-            for (int q = b; q < e; ++q) {
-                const float2 ah = Ah[q], al = Al[q];
-                const float4 xh = Xh[(int64_t)col[q] * h + c];
+            auto mac = [&](float2 ah, float2 al, float4 xh) {
                 const float2 rh = both(ah.x), nrh = both(-ah.x), rl = both(al.x);
                 const float2 ih = both(ah.y), nih = both(-ah.y), il = both(al.y);
                 df_mac1_2(a0, make_float2(xh.x, xh.y), rh, nrh, rl);
                 df_mac1_2(a1, make_float2(xh.z, xh.w), rh, nrh, rl);
                 df_mac1_2(a0, make_float2(-xh.y, xh.x), ih, nih, il);
                 df_mac1_2(a1, make_float2(-xh.w, xh.z), ih, nih, il);
+            };
+            int q = b;
+            for (; q + 1 < e; q += 2) {  // two entries' loads in flight together
+                const float2 ah0 = Ah[q], al0 = Al[q], ah1 = Ah[q + 1], al1 = Al[q + 1];
+                const float4 x0 = Xh[(int64_t)col[q] * h + c], x1 = Xh[(int64_t)col[q + 1] * h + c];
+                mac(ah0, al0, x0);
+                mac(ah1, al1, x1);
             }
+            if (q < e) mac(Ah[q], Al[q], Xh[(int64_t)col[q] * h + c]);
             a0 = df_norm_2(a0);
             a1 = df_norm_2(a1);
             Wh[row * h + c] = make_float4(a0.h.x, a0.h.y, a1.h.x, a1.h.y);
@@ -860,11 +867,20 @@ __global__ void __launch_bounds__(256) dcgs_update_df_kernel(int64_t nm, int m, 
     }
 }
 
+constexpr int kUpdRing = 4;
+constexpr int kUpdSmem = kUpdRing * 4 * 256 * 16;
+
+__device__ __forceinline__ void copy16(float4* dst, const float4* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
 // The same pass for an even m, bound by memory (16 k + 64 bytes per element): a
 // thread takes two adjacent columns (16-byte accesses) of two rows, so that the
-// coefficients and their packed forms serve both, and has the next basis vector
-// on its way while it works on one.  A block is (column pairs) x (rows), rows
-// contiguous in memory.  With one column of one row per thread the Arnoldi steps
+// coefficients and their packed forms serve both, and has the next three basis
+// vectors on their way into shared memory (its own places, no barrier) while it
+// works on one: registers for as many bytes in flight would leave too few
+// threads.  A block is (column pairs) x (rows), rows contiguous in memory.  With one column of one row per thread the Arnoldi steps
 // of a solve (458,220 rows, 32 columns, 24 steps, dot products included) took
 // 25.8 ms, now 24.0.
 __global__ void __launch_bounds__(256) dcgs_update_df2_kernel(int64_t n, int h, int k, float4* __restrict__ V,
@@ -883,9 +899,23 @@ __global__ void __launch_bounds__(256) dcgs_update_df2_kernel(int64_t n, int h, 
     float4* const vk = V + (int64_t)k * vstride;
     struct Pair { float4 h[2], l[2]; };  // two columns of the two rows
     auto load = [&](const float4* p) { return Pair{{p[e0], p[e1]}, {p[nh + e0], p[nh + e1]}}; };
+    extern __shared__ __align__(16) float4 ring[];  // [kUpdRing][4][256]
+    float4* const mine = ring + threadIdx.y * blockDim.x + threadIdx.x;
+    auto fetch = [&](int i) {
+        if (i < k) {
+            const float4* p = V + (int64_t)i * vstride;
+            float4* d = mine + (i % kUpdRing) * 4 * 256;
+            copy16(d, p + e0);
+            copy16(d + 256, p + e1);
+            copy16(d + 512, p + nh + e0);
+            copy16(d + 768, p + nh + e1);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int i = 0; i < kUpdRing - 1; ++i) fetch(i);
     auto lo2 = [](float4 v, int c) { return c ? make_float2(v.z, v.w) : make_float2(v.x, v.y); };
     const Pair v = load(vk), w = load(W);
-    Pair next = k > 0 ? load(V) : v;
     dfl2 q[2][2], x[2][2];  // [column][row]: q_k and v_{k+1}
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
@@ -901,8 +931,10 @@ __global__ void __launch_bounds__(256) dcgs_update_df2_kernel(int64_t n, int h, 
         }
     }
     for (int i = 0; i < k; ++i) {
-        const Pair u = next;
-        if (i + 1 < k) next = load(V + (int64_t)(i + 1) * vstride);
+        fetch(i + kUpdRing - 1);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kUpdRing - 1) : "memory");
+        const float4* const d = mine + (i % kUpdRing) * 4 * 256;
+        const Pair u = {{d[0], d[256]}, {d[512], d[768]}};
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             const float4 a = coefQ[i * m + 2 * cp + c], b = coefW[i * m + 2 * cp + c];
@@ -1089,6 +1121,13 @@ void GmresDF::norms2(const float2* xh, double* out, cudaStream_t st) {
     MWI_CHECK_LAUNCH();
 }
 
+static void allow_update_smem() {
+    static std::once_flag once;
+    std::call_once(once, [] {
+        MWI_CUDA(cudaFuncSetAttribute(dcgs_update_df2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUpdSmem));
+    });
+}
+
 int GmresDF::cycle(const OpA& A, const OpM& M, const float2* r0, float2* x, const double* tol, int max_steps,
                    cudaStream_t st, int* iters_used) {
     const int64_t nm = n * m;
@@ -1131,7 +1170,8 @@ int GmresDF::cycle(const OpA& A, const OpM& M, const float2* r0, float2* x, cons
             MWI_CHECK_LAUNCH();
             if (m % 2 == 0) {
                 const int h = m / 2, hx = std::min(h, 256), hy = 256 / hx;
-                dcgs_update_df2_kernel<<<dim3(nblocks(n, 2 * hy), (h + hx - 1) / hx), dim3(hx, hy), 0, st>>>(
+                allow_update_smem();
+                dcgs_update_df2_kernel<<<dim3(nblocks(n, 2 * hy), (h + hx - 1) / hx), dim3(hx, hy), kUpdSmem, st>>>(
                     n, h, k, reinterpret_cast<float4*>(V.p), vs / 2, reinterpret_cast<const float4*>(W.p), hdf.p,
                     hdf2.p, scal.p, last ? 0 : 1);
             } else {
