@@ -198,53 +198,34 @@ __global__ void __launch_bounds__(128, 3) panel_rows_kernel(const int2* __restri
         }
     }
     __syncthreads();
-    if (tl.y < 0) {
-        const int c = -1 - tl.y + threadIdx.x;
-        if (c >= k) return;
-        C* X = F + (int64_t)c * f + k;
-        C x[NB];
+    const bool left = tl.y < 0;
+    const int64_t i = left ? -1 - tl.y + threadIdx.x : tl.y + threadIdx.x;
+    if (i >= (left ? k : f)) return;
+    // a row's entries of the step's columns, or a column's of the step's rows, all
+    // loads in flight together, then W times them in place
+    C* const X = left ? F + i * f + k : F + k * f + i;
+    const int64_t step = left ? 1 : f;
+    C x[NB];
 #pragma unroll
-        for (int r = 0; r < NB; ++r) x[r] = r < nb ? X[r] : czero<C>();
+    for (int j = 0; j < NB; ++j) x[j] = j < nb ? X[j * step] : czero<C>();
 #pragma unroll
-        for (int r = NB - 1; r > 0; --r)
+    for (int j = NB - 1; j > 0; --j)
 #pragma unroll
-            for (int q = 0; q < NB; ++q)
-                if (q < r) {
-                    x[r] = cfma(W[r][q], x[q], x[r]);
-                    if (q % 8 == 7) __syncwarp();
-                }
+        for (int q = 0; q < NB; ++q)
+            if (q < j) {
+                x[j] = cfma(W[j][q], x[q], x[j]);
+                if (q % 8 == 7) __syncwarp();
+            }
+    if (left) {
 #pragma unroll
-        for (int r = 0; r < NB; ++r)
-            if (r < nb) X[r] = x[r];
-        return;
+        for (int j = 0; j < NB; ++j)
+            if (j < nb) X[j] = x[j];
+    } else {
+        C* const L = lbuf + l_off[s] + k * f + i;
+#pragma unroll
+        for (int j = 0; j < NB; ++j)
+            if (j < nb) L[j * f] = cmul(x[j], W[j][j]);
     }
-    const int64_t i = (int64_t)tl.y + threadIdx.x;
-    if (i >= f) return;
-    C* L = lbuf + l_off[s] + (int64_t)k * f + i;
-    // the row's products accumulate in registers while its entries stream in,
-    // eight independent loads at a time
-    C acc[NB];
-#pragma unroll
-    for (int j = 0; j < NB; ++j) acc[j] = czero<C>();
-#pragma unroll
-    for (int c0 = 0; c0 < NB; c0 += 8) {
-        C a[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) a[q] = c0 + q < nb ? F[(int64_t)(k + c0 + q) * f + i] : czero<C>();
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            acc[c0 + q] = cadd(acc[c0 + q], a[q]);
-#pragma unroll
-            for (int j = 0; j < NB; ++j)
-                if (j > c0 + q) {
-                    acc[j] = cfma(a[q], W[j][c0 + q], acc[j]);
-                    if (j % 8 == 7) __syncwarp();
-                }
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < NB; ++j)
-        if (j < nb) L[(int64_t)j * f] = cmul(acc[j], W[j][j]);
 }
 
 // The products of the step (k >= 0, one step's pivots) and of the level's end
