@@ -45,6 +45,25 @@ struct Gmres {
     }
 };
 
+// The status of an Arnoldi step on its way to the host: a pinned buffer, so that
+// the copy does not hold up the launches behind it, and the event that says it
+// has arrived.
+struct StepStatus {
+    int* host = nullptr;
+    cudaEvent_t ready = nullptr;
+    StepStatus() = default;
+    StepStatus(const StepStatus&) = delete;
+    StepStatus& operator=(const StepStatus&) = delete;
+    ~StepStatus() {
+        if (host) cudaFreeHost(host);
+        if (ready) cudaEventDestroy(ready);
+    }
+    void create() {
+        if (!host) MWI_CUDA(cudaMallocHost((void**)&host, 2 * sizeof(int)));
+        if (!ready) MWI_CUDA(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
+    }
+};
+
 // FGMRES whose FP64-quality vectors (basis V, w, residual, iterate) are
 // double-float planes (hi [n][m] float2 followed by lo [n][m] float2) and
 // whose preconditioned directions Z are complex FP32 (the preconditioner's
@@ -66,6 +85,7 @@ struct GmresDF {
     DevBuf<double2> H, Hp, cs, sn, g, y, h, partial;
     DevBuf<double> dvec;
     DevBuf<int> ivec;
+    StepStatus status;
     std::function<void(int, const std::function<void()>&)> timer;
 
     void reserve(int64_t n, int m, int restart);

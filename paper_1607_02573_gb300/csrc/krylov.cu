@@ -8,6 +8,7 @@
 // Orthogonalisation is classical Gram-Schmidt applied twice (CGS2): dots of
 // all basis vectors with w in one pass, then one fused update pass.
 #include <algorithm>
+#include <cstring>
 #include <mutex>
 #include <type_traits>
 
@@ -475,8 +476,9 @@ __global__ void __launch_bounds__(256) spmm_df_kernel(int64_t n, const int32_t* 
 // same bit for bit.
 // w = A z (RES = false): the error-free products and sums bound it; they run on
 // (re, im) pairs, two operations per instruction.  458,220 rows, 7.35 M entries,
-// ms per product: 32 columns 0.48 -> 0.45, 31 columns (one per lane, 32 lanes a
-// row instead of four passes of 8) 0.57 -> 0.46, 6 columns 0.156 -> 0.126.
+// ms per product: 32 columns 0.48 -> 0.45, with two entries' loads in flight
+// 0.41; 31 columns (one per lane, 32 lanes a row instead of four passes of 8)
+// 0.57 -> 0.46; 6 columns 0.156 -> 0.115.
 template <int G, bool RES>
 __global__ void __launch_bounds__(256) spmm_df2_kernel(int64_t n, const int32_t* __restrict__ rp,
                                                        const int32_t* __restrict__ col, const float2* __restrict__ Ah,
@@ -751,6 +753,8 @@ __global__ void arnoldi_dcgs_kernel(int m, int k, int restart, int last, const d
                                     double* __restrict__ resid, double* __restrict__ rho,
                                     int* __restrict__ n_active, float4* __restrict__ coefQ,
                                     float4* __restrict__ coefW, float4* __restrict__ scal) {
+    // n_active[0]: columns still active; n_active[1]: the largest of their residuals
+    // over their tolerances, as the bits of a float (non-negative, so ordered alike)
     const int c = blockIdx.x, lane = threadIdx.x;
     const int nq = k;
     const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -808,8 +812,12 @@ __global__ void arnoldi_dcgs_kernel(int m, int k, int restart, int last, const d
         resid[c] = rr;
         rho[c] = rk;
         kcol[c] = stop ? k + 1 : k;
-        if (stop && !last) active[c] = 0;
-        else if (!stop || !(rr <= tol[c])) atomicAdd(n_active, 1);
+        if (stop && !last) {
+            active[c] = 0;
+        } else if (!stop || !(rr <= tol[c])) {
+            atomicAdd(n_active, 1);
+            atomicMax(n_active + 1, __float_as_int(fminf((float)(rr / tol[c]), 3e38f)));
+        }
     }
     // fused update: q_k = v_k / nu - sum_i q_i a_i / nu;
     // v_{k+1} = w / rho_k - sum_i q_i (b_i - a_i c_k / nu) / rho_k - v_k c_k / (nu rho_k)
@@ -880,9 +888,10 @@ __device__ __forceinline__ void copy16(float4* dst, const float4* src) {
 // coefficients and their packed forms serve both, and has the next three basis
 // vectors on their way into shared memory (its own places, no barrier) while it
 // works on one: registers for as many bytes in flight would leave too few
-// threads.  A block is (column pairs) x (rows), rows contiguous in memory.  With one column of one row per thread the Arnoldi steps
-// of a solve (458,220 rows, 32 columns, 24 steps, dot products included) took
-// 25.8 ms, now 24.0.
+// threads.  A block is (column pairs) x (rows), rows contiguous in memory.  With
+// one column of one row per thread the Arnoldi steps of a solve (458,220 rows, 32
+// columns, 24 steps, dot products included) took 25.8 ms; two by two with the
+// next vector in registers 24.0; now 22.8.
 __global__ void __launch_bounds__(256) dcgs_update_df2_kernel(int64_t n, int h, int k, float4* __restrict__ V,
                                                               int64_t vstride, const float4* __restrict__ W,
                                                               const float4* __restrict__ coefQ,
@@ -1145,14 +1154,16 @@ int GmresDF::cycle(const OpA& A, const OpM& M, const float2* r0, float2* x, cons
     // v_0 = r0 / beta exactly (q_0 = v_0: no reorthogonalisation at step 0)
     scale_df_kernel<<<nblocks(nm, 256), 256, 0, st>>>(nm, m, r0, invdf.p, V.p);
     MWI_CHECK_LAUNCH();
+    status.create();
     int k = 0;
-    int n_active_host = 1;
+    bool ahead = false;   // z_k has been launched with the step before
+    float left = 0.f, left_before = 0.f;  // largest residual over tolerance after this step and the one before
     for (; k < max_steps; ++k) {
         float2* vk = V.p + (int64_t)k * vs;
         float2* zk = Z.p + (int64_t)k * nm;
         // the preconditioner sees the FP32 head of v_k (once orthogonalised);
         // z_k is stored exactly
-        M(vk, zk);
+        if (!ahead) M(vk, zk);
         A(zk, W.p);
         const int last = k + 1 == max_steps ? 1 : 0;
         auto ortho = [&] {
@@ -1164,10 +1175,12 @@ int GmresDF::cycle(const OpA& A, const OpM& M, const float2* r0, float2* x, cons
             const int nout = 2 * k + 3;
             dots_reduce_kernel<<<nout, 1024, 0, st>>>(nblk, nout, 0, m, partial.p, h.p, nullptr, nullptr);
             MWI_CHECK_LAUNCH();
-            MWI_CUDA(cudaMemsetAsync(nact, 0, sizeof(int), st));
+            MWI_CUDA(cudaMemsetAsync(nact, 0, 2 * sizeof(int), st));
             arnoldi_dcgs_kernel<<<m, 32, 0, st>>>(m, k, restart, last, h.p, H.p, Hp.p, cs.p, sn.p, g.p, active, kcol,
                                                   tol, resid, rho, nact, hdf.p, hdf2.p, scal.p);
             MWI_CHECK_LAUNCH();
+            MWI_CUDA(cudaMemcpyAsync(status.host, nact, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+            MWI_CUDA(cudaEventRecord(status.ready, st));
             if (m % 2 == 0) {
                 const int h = m / 2, hx = std::min(h, 256), hy = 256 / hx;
                 allow_update_smem();
@@ -1182,9 +1195,16 @@ int GmresDF::cycle(const OpA& A, const OpM& M, const float2* r0, float2* x, cons
         };
         if (timer) timer(2, ortho);
         else ortho();
-        MWI_CUDA(cudaMemcpyAsync(&n_active_host, nact, sizeof(int), cudaMemcpyDeviceToHost, st));
-        MWI_CUDA(cudaStreamSynchronize(st));
-        if (n_active_host == 0) { ++k; break; }
+        // The next preconditioner application is launched before this step's status
+        // has come back if the last step's reduction of the residual, twice over,
+        // would still leave it above the tolerance: the GPU then has work while the
+        // host waits and launches (12 us a step).  A wrong guess costs one application.
+        ahead = !last && k > 0 && left_before > 0.f && left * (left / left_before) * (left / left_before) > 1.f;
+        if (ahead) M(V.p + (int64_t)(k + 1) * vs, Z.p + (int64_t)(k + 1) * nm);
+        MWI_CUDA(cudaEventSynchronize(status.ready));
+        left_before = left;
+        std::memcpy(&left, status.host + 1, sizeof(float));
+        if (status.host[0] == 0) { ++k; break; }
     }
     launch_lsq(m, restart, H.p, g.p, kcol, y.p, ydf.p, st);
     lincomb_df_kernel<<<nblocks(nm, 256), 256, 0, st>>>(nm, m, k, Z.p, nm, ydf.p, x);
