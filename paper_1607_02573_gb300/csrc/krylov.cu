@@ -132,7 +132,8 @@ __global__ void __launch_bounds__(256) dots_kernel(int64_t n, int m, int nvec_in
 }
 
 // h[i][c] = sum_b partial[b][i][c] for i < nvec; hacc[i][c] += h[i][c] for i < nacc;
-// hdf (optional) receives h as double-floats (re hi, re lo, im hi, im lo).
+// hdf (optional) receives h as double-floats (re hi, re lo, im hi, im lo); clear
+// (optional): two counters set to zero on the way.
 // One block per vector index i: 32 warps split the blocks b (b = warp, warp +
 // 32, ...), lanes over columns, then a fixed-order sum of the 32 partial sums.
 // The chain of loads and FP64 additions per warp bounds it (with 8 warps a
@@ -140,9 +141,10 @@ __global__ void __launch_bounds__(256) dots_kernel(int64_t n, int m, int nvec_in
 __global__ void __launch_bounds__(1024) dots_reduce_kernel(int nblk, int nvec, int nacc, int m,
                                                           const double2* __restrict__ partial,
                                                           double2* __restrict__ h, double2* __restrict__ hacc,
-                                                          float4* __restrict__ hdf) {
+                                                          float4* __restrict__ hdf, int* __restrict__ clear) {
     __shared__ double2 red[32][33];
     const int i = blockIdx.x;
+    if (clear && i == 0 && threadIdx.x < 2) clear[threadIdx.x] = 0;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     for (int c0 = 0; c0 < m; c0 += 32) {
         const int c = c0 + tx;
@@ -1014,7 +1016,7 @@ static void dots_launch(int64_t n, int m, const C* Vb, int nvec, int64_t vstride
     dots_kernel<C><<<grd, blk, 0, st>>>(n, m, nvec, Vb, vstride, w, self, partial);
     MWI_CHECK_LAUNCH();
     const int nt = nvec + self;
-    dots_reduce_kernel<<<nt, 1024, 0, st>>>(kDotBlocks, nt, nvec, m, partial, out, acc, hdf);
+    dots_reduce_kernel<<<nt, 1024, 0, st>>>(kDotBlocks, nt, nvec, m, partial, out, acc, hdf, nullptr);
     MWI_CHECK_LAUNCH();
 }
 
@@ -1173,9 +1175,8 @@ int GmresDF::cycle(const OpA& A, const OpM& M, const float2* r0, float2* x, cons
             dots2_kernel<<<grd, blk, 0, st>>>(n, m, k, V.p, vs, vk, W.p, partial.p);
             MWI_CHECK_LAUNCH();
             const int nout = 2 * k + 3;
-            dots_reduce_kernel<<<nout, 1024, 0, st>>>(nblk, nout, 0, m, partial.p, h.p, nullptr, nullptr);
+            dots_reduce_kernel<<<nout, 1024, 0, st>>>(nblk, nout, 0, m, partial.p, h.p, nullptr, nullptr, nact);
             MWI_CHECK_LAUNCH();
-            MWI_CUDA(cudaMemsetAsync(nact, 0, 2 * sizeof(int), st));
             arnoldi_dcgs_kernel<<<m, 32, 0, st>>>(m, k, restart, last, h.p, H.p, Hp.p, cs.p, sn.p, g.p, active, kcol,
                                                   tol, resid, rho, nact, hdf.p, hdf2.p, scal.p);
             MWI_CHECK_LAUNCH();
