@@ -402,6 +402,11 @@ void factorize_fronts(const FrontsDev& F, const UpdateTiles& ut, const double2* 
     MWI_REQUIRE(ut.nb == NB && ut.tile == TILE, MWI_EINVAL, "internal: update tiles built for another blocking");
     MWI_CUDA(cudaMemsetAsync(ws, 0, (size_t)(F.ws_entries + F.nloc) * sizeof(C), st));
     const int nlev = (int)F.level_ptr.size() - 1;
+    // the largest front this factorisation accepts, unchanged: 12,800 rows in
+    // complex FP32, 6,400 in FP64
+    for (int l = 0; l < nlev; ++l)
+        MWI_REQUIRE(2 * (size_t)F.level_fmax[l] * sizeof(C) <= 200 * 1024, MWI_EINVAL,
+                    "front too large (" + std::to_string(F.level_fmax[l]) + " rows)");
     size_t range = 0, ext = 0, end = 0;
     for (int l = 0; l < nlev; ++l) {
         const int lo0 = F.level_ptr[l], hi = F.level_ptr[l + 1];
