@@ -504,7 +504,7 @@ void upload_fronts(const Decomposition& D, FrontsDev& F, cudaStream_t st) {
     F.sch_entries[0] = D.sch_entries[0];
     F.sch_entries[1] = D.sch_entries[1];
     F.n_sub = D.n_sub;
-    // GEMM tile lists of the sweeps and per-level offsets of the inverse scratch
+    // GEMM tile lists of the sweeps
     for (int pass = 0; pass < 2; ++pass) {
         TileLists& TL = pass == 0 ? F.tiles64 : F.tiles32;
         TL.tm = sweep_tile_rows(pass == 0);

@@ -5,8 +5,8 @@
 // products accumulated in tensor memory.
 //
 // Factor layout ("tiled panels", written once per factorisation by
-// pack_tiled_kernel).  The TF32 form of tcgen05.mma reads both operands
-// K-major (K contiguous in a line), and the two sweeps contract a front's
+// pack_tiled_kernel).  The A operand is K-major (K contiguous in a line), and the
+// two sweeps contract a front's
 // f x p partitioned-inverse panel [L11^{-1}; -L21 L11^{-1}] over different
 // indices -- the forward product over pivots, the backward one over rows --
 // so the panel is stored twice, cut into 8 x 8 blocks (rows and pivots padded
@@ -42,7 +42,7 @@
 // list, so it is done or being done by a running CTA whatever the number of
 // CTAs that run at the same time:
 //   - forward tile of a front: all forward tiles of its children, counted per
-//     front by the epilogues (release) and polled by the copy warp (acquire);
+//     front by the epilogues (release) and polled by the gather warps (acquire);
 //   - backward tile: all backward tiles of the parent (of the root: its own
 //     forward tiles), which closes the chain over everything else it reads.
 // The children add their update rows straight into the parent's pivot rows in
