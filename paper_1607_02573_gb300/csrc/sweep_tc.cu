@@ -42,7 +42,8 @@
 // list, so it is done or being done by a running CTA whatever the number of
 // CTAs that run at the same time:
 //   - forward tile of a front: all forward tiles of its children, counted per
-//     front by the epilogues (release) and polled by the gather warps (acquire);
+//     front by the epilogues (release) and polled by the gather warps (acquire),
+//     which hand the order on to their other lanes and to the tile's epilogue;
 //   - backward tile: all backward tiles of the parent (of the root: its own
 //     forward tiles), which closes the chain over everything else it reads.
 // The children add their update rows straight into the parent's pivot rows in
@@ -107,6 +108,7 @@ constexpr int kThreads = 288;
 constexpr int kTmemCols = 256;
 constexpr int kSmemBytes =
     kStages * kStage + 1024 /* barriers */ + kRing * 128 + kSurBufs * kUrCache * 4 + 1024 /* alignment */;
+static_assert((3 * kStages + 4 + 2 * kRing + kSurBufs + 1) * 8 + 8 <= 1024, "barriers");
 static_assert(kSmemBytes * kCtasPerSm <= 228 * 1024 - 2048, "shared memory per SM");
 constexpr long long kWaitLimit = 1ll << 24;
 constexpr int kDepLimit = 1 << 22;          // polls of a dependency count (a few seconds)
@@ -235,8 +237,8 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 __device__ __forceinline__ void red_release(int* p) {
     asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p) : "memory");
 }
-// bounded wait until *cnt >= target (one lane); false if the CTA aborts, another
-// CTA has reported an error or the limit expires
+// bounded wait until *cnt >= target (one lane; dep_wait_warp for all); false if the
+// CTA aborts, another CTA has reported an error or the limit expires
 __device__ __forceinline__ bool dep_wait(const int* cnt, int target, volatile int* abort_flag, int* err, int code) {
     for (int it = 0; it < kDepLimit; ++it) {
         if (ld_acquire(cnt) >= target) return true;
@@ -252,6 +254,16 @@ __device__ __forceinline__ bool dep_wait(const int* cnt, int target, volatile in
     *abort_flag = 1;
     atomicExch(err, code);
     return false;
+}
+// The same for a whole warp: each lane polls its own count (cnt = nullptr: none).
+// A vote does not order memory; the __syncwarp() is what orders the other lanes'
+// reads after a lane's acquire.
+__device__ __forceinline__ bool dep_wait_warp(const int* cnt, int target, volatile int* abort_flag, int* err,
+                                              int code) {
+    const bool ok = !cnt || dep_wait(cnt, target, abort_flag, err, code);
+    const bool all = __all_sync(0xffffffffu, ok);
+    __syncwarp();
+    return all;
 }
 
 // Tile geometry shared by every role.  Forward: M = front rows row0..
@@ -320,8 +332,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStage);
     // bars: raw[kStages] (panel blocks landed), rows[kStages] (right-hand-side rows
     // landed), empty[kStages] (stage consumed), tfull[2], tempty[2], tile[kRing]
-    // (descriptor written), sur[kSurBufs], begun (tile begun)
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * kStages + 4 + kRing + kSurBufs + 1);
+    // (descriptor written), sur[kSurBufs], begun (tile begun), deps[kRing] (the tile's
+    // dependencies are met)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * kStages + 4 + 2 * kRing + kSurBufs + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     RingSlot* ring = reinterpret_cast<RingSlot*>(smem + kStages * kStage + 1024);
     int32_t* sur = reinterpret_cast<int32_t*>(smem + kStages * kStage + 1024 + kRing * 128);
@@ -336,6 +349,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
     auto tile_par = [&](int it) { return (uint32_t)(it / kRing) & 1; };
     auto sur_bar = [&](int b) { return smem_u32(bars + 3 * kStages + 4 + kRing + b); };
     const uint32_t begun_bar = smem_u32(bars + 3 * kStages + 4 + kRing + kSurBufs);
+    auto deps_bar = [&](int it) {
+        return smem_u32(bars + 3 * kStages + 4 + kRing + kSurBufs + 1 + (it & (kRing - 1)));
+    };
 
     // stale shared memory must be finite: the MMA reads whole 128-row groups of
     // panel blocks, and the columns and rows without data go nowhere
@@ -354,6 +370,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
         }
         for (int b = 0; b < kSurBufs; ++b) mbar_init(sur_bar(b), 1);
         for (int b = 0; b < kRing; ++b) mbar_init(tile_bar(b), 1);
+        for (int b = 0; b < kRing; ++b) mbar_init(deps_bar(b), 1);
         mbar_init(begun_bar, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -461,13 +478,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                 iu = sur + (nsur % kSurBufs) * kUrCache + (slot->d.u_off & 3);
                 ++nsur;
             }
-            // the rows are other tiles' results
-            if (lane < 2) {
-                const int dep = lane == 0 ? slot->d.dep0 : slot->d.dep1;
-                if (dep >= 0)
-                    ok = dep_wait(cnt + dep, (lane == 0 ? slot->d.need0 : slot->d.need1) * nchunks, abort_flag, err, 7);
-            }
-            if (!(ok = __all_sync(0xffffffffu, ok))) break;
+            // the rows are other tiles' results; the epilogue, which reads such rows
+            // as well, learns from warp 2 that they are there
+            const int dep = lane == 0 ? slot->d.dep0 : (lane == 1 ? slot->d.dep1 : -1);
+            const int need = lane == 0 ? slot->d.need0 : slot->d.need1;
+            if (!(ok = dep_wait_warp(dep >= 0 ? cnt + dep : nullptr, need * nchunks, abort_flag, err, 7))) break;
+            if (warp == 2 && lane == 0) mbar_arrive(deps_bar(it));
             for (int st = 0; st < G.nst; ++st, ++g) {
                 const int s = (int)(g % kStages);
                 const uint32_t ph = (uint32_t)((g / kStages) & 1);
@@ -564,11 +580,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             }
             if (d.sib >= 0 && __any_sync(0xffffffffu, add)) {
                 // the second child adds to the parent's rows after the first
-                if (lane == 0) ok = dep_wait(cnt + d.sib, d.needs * nchunks, abort_flag, err, 9);
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (!ok) break;
+                if (!(ok = dep_wait_warp(lane == 0 ? cnt + d.sib : nullptr, d.needs * nchunks, abort_flag, err, 9)))
+                    break;
             }
             if (!(ok = mbar_wait(tfull_bar(buf), (it >> 1) & 1, abort_flag, err, 5))) break;
+            // past already (the product came after it): orders this lane's reads of the
+            // children's rows after the gather warp's acquire
+            if (!(ok = mbar_wait(deps_bar(it), tile_par(it), abort_flag, err, 11))) break;
             tc_fence_after();
             const uint32_t t0 = tmem + ((uint32_t)(lg * 32) << 16) + buf * 128;
             // whole 32-byte accesses: a lane's row is a line of its own, so an access

@@ -1,0 +1,49 @@
+"""The one-launch tensor-core sweeps (sweep_engine 4): what their tiles hand to
+each other inside the launch, their rounding, and their bounded waits.
+"""
+
+import numpy as np
+import pytest
+
+from tests._helpers import FREQ, chamber_case
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1607_02573_gb300 import mwi
+    return mwi
+
+
+@pytest.fixture(scope="module")
+def chamber(lib):
+    mesh, eps, _, _ = chamber_case(12, 11)
+    return lib.Mesh(mesh.xyz, mesh.tet, mesh.bface_tag), eps
+
+
+def _block(n, m, seed):
+    rng = np.random.default_rng(seed)
+    return torch.from_numpy(rng.standard_normal((n, m)) + 1j * rng.standard_normal((n, m))).cuda()
+
+
+@pytest.mark.parametrize("n_sub,leaf,m", [(1, 9, 68), (7, 33, 96), (7, 128, 31)])
+def test_repeated_applications_agree_bit_for_bit(lib, chamber, n_sub, leaf, m):
+    """A tile reads rows that other tiles of the launch have just written; the
+    sums have a fixed order, so a read that came too early would show as a
+    difference between applications.  Deep trees, one to three column chunks;
+    every chunk also as a block of its own."""
+    M, eps = chamber
+    P = lib.Problem(M, eps, FREQ, n_sub=n_sub, precision=1, nd_leaf=leaf)
+    X = _block(M.ndof, m, 5)
+    ref = P.oras_apply(X).cpu()
+    assert torch.isfinite(torch.view_as_real(ref)).all()
+    for _ in range(12):
+        assert torch.equal(P.oras_apply(X).cpu(), ref)
+    for c in range(0, m, 32):
+        assert torch.equal(P.oras_apply(X[:, c:c + 32].contiguous()).cpu(), ref[:, c:c + 32])
+    P.close()
