@@ -53,7 +53,8 @@ typedef enum {
     MWI_ENOMEM = 2,     /* host or device allocation failed */
     MWI_ENOTCONV = 3,   /* FGMRES hit max_iter before rtol on some column */
     MWI_ECUDA = 4,      /* a CUDA runtime call failed */
-    MWI_ETIMEOUT = 5,   /* reserved: bounded wait expired */
+    MWI_ETIMEOUT = 5,   /* a wait inside the tensor-core sweeps' launch expired; the outputs are
+                           not valid, the problem stays usable */
     MWI_ESTATE = 6,     /* call out of order (e.g. gradient before forward) */
     MWI_ESINGULAR = 7   /* a zero pivot could not be perturbed */
 } mwi_status;
@@ -339,6 +340,13 @@ mwi_status mwi_oras_traffic(mwi_problem_t prob, int32_t m, double* bytes);
  * the mesh and its decomposition, shared by the problems on that mesh, are not
  * counted.  For admission against a memory budget (a serving cache). */
 mwi_status mwi_problem_device_bytes(mwi_problem_t prob, int64_t* bytes);
+
+/* How often a tile of the tensor-core sweeps (sweep_engine 4) looks for the
+ * results of the tiles it depends on before the launch gives up and the call
+ * returns MWI_ETIMEOUT: polls >= 0, or < 0 for the default (about four
+ * million, a few seconds).  0 lets every such wait expire at once.  Failure
+ * detection; no counterpart in the paper. */
+mwi_status mwi_set_sweep_polls(mwi_problem_t prob, int32_t polls);
 
 /* Per tree level of the multifrontal sweeps (deepest level first; a
  * measurement aid, no counterpart in the paper): *n_levels levels; for the

@@ -169,6 +169,7 @@ struct mwi_problem {
     DevBuf<float> wt;        // tiled, swizzled copy of the c64 panels (tensor-core sweeps)
     DevBuf<int> sweep_err;   // error code of the tensor-core sweeps' bounded waits
     DevBuf<int> sweep_cnt;   // their completion counts (one application at a time: the problem's stream)
+    int sweep_polls = kSweepPolls;
     DevBuf<int> perturbed;
     int n_perturbed = 0;
     // solve state
@@ -287,6 +288,7 @@ SweepCfg sweep_cfg(const mwi_problem* P) {
     c.wt = P->wt.p;
     c.err = P->sweep_err.p;
     c.cnt = P->sweep_cnt.p;
+    c.polls = P->sweep_polls;
     return c;
 }
 
@@ -1647,6 +1649,13 @@ mwi_status mwi_oras_apply_device_noalloc(mwi_problem_t P, const double* x_dev, d
                            sweep_cfg(P));
         MWI_CUDA(cudaStreamSynchronize(P->st));
         check_sweep_error(P);
+    });
+}
+
+mwi_status mwi_set_sweep_polls(mwi_problem_t P, int32_t polls) {
+    return guard([&] {
+        MWI_REQUIRE(P, MWI_EINVAL, "null problem");
+        P->sweep_polls = polls < 0 ? kSweepPolls : polls;
     });
 }
 

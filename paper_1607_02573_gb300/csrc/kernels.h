@@ -169,12 +169,15 @@ void factorize_fronts(const FrontsDev& F, const UpdateTiles& ut, const double2* 
 
 // Complex FP32 sweep engine: tc = 0 CUDA cores, 1 mma.sync 3xTF32, 2 mma.sync
 // TF32, 4 tcgen05 TF32 over the tiled panel store wt (cnt: FrontsDev::tc_counts()
-// ints of the caller's, used by one application at a time; err: the kernels'
-// bounded-wait error code, 0 = none)
+// ints of the caller's, used by one application at a time; polls: looks at a count
+// before a tile's wait for other tiles gives up; err: the kernels' bounded-wait
+// error code, 0 = none)
+constexpr int kSweepPolls = 1 << 22;  // a few seconds
 struct SweepCfg {
     int tc = 0;
     const float* wt = nullptr;
     int* cnt = nullptr;
+    int polls = kSweepPolls;
     int* err = nullptr;
 };
 
@@ -196,7 +199,7 @@ int64_t tiled_panel_floats(int p, int f);
 void pack_tiled(const int2* blocks, int64_t nblocks, const int64_t* f_off, const int64_t* t_off, const int32_t* P,
                 const int32_t* U, const float2* ws, float* wt, int64_t bwd_base, cudaStream_t st);
 void sweep_tc_solve(const FrontsDev& F, int m, const float* wt, const float2* dinv, float2* Y, float2* Z,
-                    float2* upd, int* cnt, int* err, cudaStream_t st);
+                    float2* upd, int* cnt, int polls, int* err, cudaStream_t st);
 
 // Allocation-free ORAS application (oras.cu): scratch from a fixed-size
 // file-scope device array of kOrasScratchBytes.

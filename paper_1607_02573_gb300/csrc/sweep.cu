@@ -612,7 +612,7 @@ void multifrontal_solve(const FrontsDev& F, const C* ws, C* Y, C* Z, C* upd, int
             // (oras_apply pads the local vectors to an even column count)
             MWI_REQUIRE(sc.wt && sc.err && sc.cnt, MWI_EINVAL, "internal: tensor-core sweeps without their buffers");
             MWI_REQUIRE((m % 2) == 0, MWI_EINVAL, "internal: tensor-core sweeps need an even column count");
-            sweep_tc_solve(F, m, sc.wt, ws + F.ws_entries, Y, Z, upd, sc.cnt, sc.err, st);
+            sweep_tc_solve(F, m, sc.wt, ws + F.ws_entries, Y, Z, upd, sc.cnt, sc.polls, sc.err, st);
             return;
         }
     }

@@ -81,7 +81,8 @@
 // even number of columns.
 // Every wait is bounded: on expiry the kernel records an error code, the other
 // roles stop at their next wait, other CTAs at their next dependency wait, and
-// the CTA frees its tensor memory and returns.
+// the CTA lets its copies and products in flight land, frees its tensor memory
+// and returns.
 #include <algorithm>
 #include <mutex>
 
@@ -111,7 +112,6 @@ constexpr int kSmemBytes =
 static_assert((3 * kStages + 4 + 2 * kRing + kSurBufs + 1) * 8 + 8 <= 1024, "barriers");
 static_assert(kSmemBytes * kCtasPerSm <= 228 * 1024 - 2048, "shared memory per SM");
 constexpr long long kWaitLimit = 1ll << 24;
-constexpr int kDepLimit = 1 << 22;          // polls of a dependency count (a few seconds)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -237,10 +237,24 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 __device__ __forceinline__ void red_release(int* p) {
     asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p) : "memory");
 }
-// bounded wait until *cnt >= target (one lane; dep_wait_warp for all); false if the
-// CTA aborts, another CTA has reported an error or the limit expires
-__device__ __forceinline__ bool dep_wait(const int* cnt, int target, volatile int* abort_flag, int* err, int code) {
-    for (int it = 0; it < kDepLimit; ++it) {
+// the same answer in every lane, so that a warp whose lanes see the abort at
+// different times leaves its loop as one (its warp-wide instructions need them all)
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err,
+                                               int code) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, err, code));
+}
+// bounded wait without the abort: for what is in flight when the CTA ends
+__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
+    for (int it = 0; it < (1 << 12); ++it)
+        if (mbar_try(bar, parity)) break;
+}
+
+// bounded wait until *cnt >= target (one lane; dep_wait_warp for all), at most
+// `polls` looks; false if the CTA aborts, another CTA has reported an error or the
+// limit expires
+__device__ __forceinline__ bool dep_wait(const int* cnt, int target, int polls, volatile int* abort_flag, int* err,
+                                         int code) {
+    for (int it = 0; it < polls; ++it) {
         if (ld_acquire(cnt) >= target) return true;
         if (*abort_flag) return false;
         if ((it & 63) == 63) {
@@ -258,9 +272,9 @@ __device__ __forceinline__ bool dep_wait(const int* cnt, int target, volatile in
 // The same for a whole warp: each lane polls its own count (cnt = nullptr: none).
 // A vote does not order memory; the __syncwarp() is what orders the other lanes'
 // reads after a lane's acquire.
-__device__ __forceinline__ bool dep_wait_warp(const int* cnt, int target, volatile int* abort_flag, int* err,
-                                              int code) {
-    const bool ok = !cnt || dep_wait(cnt, target, abort_flag, err, code);
+__device__ __forceinline__ bool dep_wait_warp(const int* cnt, int target, int polls, volatile int* abort_flag,
+                                              int* err, int code) {
+    const bool ok = !cnt || dep_wait(cnt, target, polls, abort_flag, err, code);
     const bool all = __all_sync(0xffffffffu, ok);
     __syncwarp();
     return all;
@@ -325,7 +339,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
     const TcTile* __restrict__ tiles, int ntiles, int nchunks, int* __restrict__ cnt,
     const int32_t* __restrict__ urows, const int2* __restrict__ asm2, const int32_t* __restrict__ pdst,
     const float* __restrict__ wt, const float2* __restrict__ dinv, float2* Y, float2* Z, float2* upd, int m,
-    int* err) {
+    int polls, int* err) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                            ~(uintptr_t)1023);
@@ -391,7 +405,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
         long long g = 0;
         bool ok = true;
         for (int it = 0; ok; ++it) {
-            if (!(ok = mbar_wait(tile_bar(it), tile_par(it), abort_flag, err, 8))) break;
+            if (!(ok = mbar_wait_warp(tile_bar(it), tile_par(it), abort_flag, err, 8))) break;
             const RingSlot* slot = ring + (it & (kRing - 1));
             if (!slot->valid) break;
             const TcGeom G = tc_geom(slot->d.p, slot->d.f, slot->d.row0, slot->d.bwd != 0);
@@ -400,7 +414,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             for (int st = 0; st < G.nst; ++st, ++g) {
                 const int s = (int)(g % kStages);
                 const uint32_t ph = (uint32_t)((g / kStages) & 1);
-                if (!(ok = mbar_wait(empty_bar(s), ph ^ 1, abort_flag, err, 1))) break;
+                if (!(ok = mbar_wait_warp(empty_bar(s), ph ^ 1, abort_flag, err, 1))) break;
                 const int k0 = G.k0 + st * kKS, nk = min(kKS, G.k0 + G.nk - k0);
                 if (lane == 0) mbar_arrive_tx(raw_bar(s), a_bytes * nk);
                 __syncwarp();
@@ -410,15 +424,16 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                 if (st == 0 && lane == 0) mbar_arrive(begun_bar);
             }
         }
-        if (!ok && lane == 0)
-            // copies still in flight land before the CTA gives its shared memory back
+        // copies still in flight land before the CTA gives its shared memory back, also
+        // when this warp is through and another one has given up
+        if (lane == 0)
             for (long long q = g > kStages ? g - kStages : 0; q < g; ++q)
-                for (int it = 0; it < (1 << 12); ++it)
-                    if (mbar_try(raw_bar((int)(q % kStages)), (uint32_t)((q / kStages) & 1))) break;
+                mbar_drain(raw_bar((int)(q % kStages)), (uint32_t)((q / kStages) & 1));
     } else if (warp == 1) {
         // ---------------- tensor-core products
         if (lane == 0) {
             long long g = 0;
+            int done = 0;  // tiles multiplied
             bool ok = true;
             constexpr uint32_t kIdesc = idesc_tf32(128, 64);
             for (int it = 0; ok; ++it) {
@@ -450,7 +465,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                 }
                 if (!ok) break;
                 mma_commit(tfull_bar(buf));
+                ++done;
             }
+            // products and commits still in flight, before the tensor memory is freed
+            for (long long q = g > kStages ? g - kStages : 0; q < g; ++q)
+                mbar_drain(empty_bar((int)(q % kStages)), (uint32_t)((q / kStages) & 1));
+            for (int q = max(0, done - 2); q < done; ++q) mbar_drain(tfull_bar(q & 1), (uint32_t)(q >> 1) & 1);
         }
     } else if (warp < 4) {
         // ---------------- right-hand-side rows into the B operand: this warp's half
@@ -461,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
         int nsur = 0;
         bool ok = true;
         for (int it = 0; ok; ++it) {
-            if (!mbar_wait(tile_bar(it), tile_par(it), abort_flag, err, 8)) break;
+            if (!mbar_wait_warp(tile_bar(it), tile_par(it), abort_flag, err, 8)) break;
             const RingSlot* slot = ring + (it & (kRing - 1));
             if (!slot->valid) break;
             const TcGeom G = tc_geom(slot->d.p, slot->d.f, slot->d.row0, slot->d.bwd != 0);
@@ -473,7 +493,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             const int32_t* iu = urows + slot->d.u_off;
             const int kfirst = G.bwd ? G.row0 : 0;
             if (indices_cached(G)) {
-                if (!(ok = mbar_wait(sur_bar(nsur % kSurBufs), (uint32_t)(nsur / kSurBufs) & 1, abort_flag, err, 6)))
+                if (!(ok = mbar_wait_warp(sur_bar(nsur % kSurBufs), (uint32_t)(nsur / kSurBufs) & 1, abort_flag, err,
+                                          6)))
                     break;
                 iu = sur + (nsur % kSurBufs) * kUrCache + (slot->d.u_off & 3);
                 ++nsur;
@@ -482,7 +503,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             // as well, learns from warp 2 that they are there
             const int dep = lane == 0 ? slot->d.dep0 : (lane == 1 ? slot->d.dep1 : -1);
             const int need = lane == 0 ? slot->d.need0 : slot->d.need1;
-            if (!(ok = dep_wait_warp(dep >= 0 ? cnt + dep : nullptr, need * nchunks, abort_flag, err, 7))) break;
+            if (!(ok = dep_wait_warp(dep >= 0 ? cnt + dep : nullptr, need * nchunks, polls, abort_flag, err, 7))) break;
             if (warp == 2 && lane == 0) mbar_arrive(deps_bar(it));
             for (int st = 0; st < G.nst; ++st, ++g) {
                 const int s = (int)(g % kStages);
@@ -490,7 +511,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                 const int nv = stage_rows(G, st);
                 const int nz = min(kKRows, (nv + 7) & ~7);  // rows that the products read
                 const uint32_t R = sbase + s * kStage + kAStage + (seg >> 3) * (kKRows * 128) + (seg & 1) * 16;
-                if (!(ok = mbar_wait(empty_bar(s), ph ^ 1, abort_flag, err, 1))) break;
+                if (!(ok = mbar_wait_warp(empty_bar(s), ph ^ 1, abort_flag, err, 1))) break;
                 if (seg < (nc >> 1)) {
                     // all addresses before the copies, which the compiler keeps in order
                     // with the index loads
@@ -521,9 +542,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
         // which is of tile i - 1 - kStages or later: that tile's rows are gathered,
         // and its accumulator waited for the epilogue of the tile two before.
         int nsur = 0;  // index buffers filled so far
-        bool ok = true;
         for (int it = 0;; ++it) {
-            if (it > 0 && !(ok = mbar_wait(begun_bar, (uint32_t)(it - 1) & 1, abort_flag, err, 10))) break;
+            if (it > 0 && !mbar_wait_warp(begun_bar, (uint32_t)(it - 1) & 1, abort_flag, err, 10)) break;
             const int tk = __shfl_sync(0xffffffffu, lane == 0 ? atomicAdd(cnt, 1) : 0, 0);
             const int ti = tk / nchunks;
             RingSlot* slot = ring + (it & (kRing - 1));
@@ -546,17 +566,16 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             }
             nsur += indices_cached(G) ? 1 : 0;
         }
-        if (!ok && lane == 0)
+        if (lane == 0)
             for (int q = max(0, nsur - kSurBufs); q < nsur; ++q)
-                for (int it = 0; it < (1 << 12); ++it)
-                    if (mbar_try(sur_bar(q % kSurBufs), (uint32_t)(q / kSurBufs) & 1)) break;
+                mbar_drain(sur_bar(q % kSurBufs), (uint32_t)(q / kSurBufs) & 1);
     } else {
         // ---------------- epilogue
         const int lg = warp & 3;  // tensor-memory lane group of this warp
         const int i = lg * 32 + lane;
         bool ok = true;
         for (int it = 0; ok; ++it) {
-            if (!mbar_wait(tile_bar(it), tile_par(it), abort_flag, err, 8)) break;
+            if (!mbar_wait_warp(tile_bar(it), tile_par(it), abort_flag, err, 8)) break;
             const RingSlot* slot = ring + (it & (kRing - 1));
             if (!slot->valid) break;
             const TcTile d = slot->d;
@@ -580,13 +599,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             }
             if (d.sib >= 0 && __any_sync(0xffffffffu, add)) {
                 // the second child adds to the parent's rows after the first
-                if (!(ok = dep_wait_warp(lane == 0 ? cnt + d.sib : nullptr, d.needs * nchunks, abort_flag, err, 9)))
+                if (!(ok = dep_wait_warp(lane == 0 ? cnt + d.sib : nullptr, d.needs * nchunks, polls, abort_flag, err,
+                                         9)))
                     break;
             }
-            if (!(ok = mbar_wait(tfull_bar(buf), (it >> 1) & 1, abort_flag, err, 5))) break;
+            if (!(ok = mbar_wait_warp(tfull_bar(buf), (it >> 1) & 1, abort_flag, err, 5))) break;
             // past already (the product came after it): orders this lane's reads of the
             // children's rows after the gather warp's acquire
-            if (!(ok = mbar_wait(deps_bar(it), tile_par(it), abort_flag, err, 11))) break;
+            if (!(ok = mbar_wait_warp(deps_bar(it), tile_par(it), abort_flag, err, 11))) break;
             tc_fence_after();
             const uint32_t t0 = tmem + ((uint32_t)(lg * 32) << 16) + buf * 128;
             // whole 32-byte accesses: a lane's row is a line of its own, so an access
@@ -599,6 +619,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             // this launch have written are read past L1.
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
+                __syncwarp();  // lanes without a row left the first half early
                 float o[32];
                 {
                     float dr[32], di[32];
@@ -735,7 +756,7 @@ int sweep_tc_ctas() {
 
 // both sweeps; cnt holds F.tc_counts() zeros
 void sweep_tc_solve(const FrontsDev& F, int m, const float* wt, const float2* dinv, float2* Y, float2* Z,
-                    float2* upd, int* cnt, int* err, cudaStream_t st) {
+                    float2* upd, int* cnt, int polls, int* err, cudaStream_t st) {
     static std::once_flag attr;
     std::call_once(attr, [] {
         MWI_CUDA(cudaFuncSetAttribute(sweep_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
@@ -746,7 +767,7 @@ void sweep_tc_solve(const FrontsDev& F, int m, const float* wt, const float2* di
     if (total <= 0) return;
     const int grid = (int)std::min<int64_t>(total, sweep_tc_ctas());
     sweep_tc_kernel<<<grid, kThreads, kSmemBytes, st>>>(F.tc_tiles.p, (int)F.tc_ntiles, nchunks, cnt, F.urows.p,
-                                                        F.asm2.p, F.pdst.p, wt, dinv, Y, Z, upd, m, err);
+                                                        F.asm2.p, F.pdst.p, wt, dinv, Y, Z, upd, m, polls, err);
     MWI_CHECK_LAUNCH();
 }
 

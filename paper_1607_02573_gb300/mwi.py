@@ -80,6 +80,7 @@ _SIGS = {
     "mwi_problem_device_bytes": [_vp, _i64p],
     "mwi_problem_estimate_bytes": [_vp, C.POINTER(mwi_solver_opts), C.c_int32, _i64p],
     "mwi_recycle_from": [_vp, _vp],
+    "mwi_set_sweep_polls": [_vp, C.c_int32],
     "mwi_sweep_levels": [_vp, C.c_int32, _i32p, _i64p, _i64p, _i64p, _i64p, _i64p],
     "mwi_oras_traffic": [_vp, C.c_int32, _dp],
     "mwi_update_kappa_device": [_vp, _vp],
@@ -473,6 +474,9 @@ class Problem:
         check(st, allow=(MWI_ENOTCONV,) if allow_notconv else ())
         self.info = info
         return J.value, R.value, grad
+
+    def set_sweep_polls(self, polls):
+        check(mwi_set_sweep_polls(self.h, polls))
 
     def sweep_levels(self):
         """Per tree level (deepest first): fronts, panel entries, update rows and

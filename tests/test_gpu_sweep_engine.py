@@ -5,6 +5,7 @@ each other inside the launch, their rounding, and their bounded waits.
 import numpy as np
 import pytest
 
+from synthetic import antenna_array, ring_antennas
 from tests._helpers import FREQ, chamber_case
 
 pytestmark = pytest.mark.gpu
@@ -46,4 +47,25 @@ def test_repeated_applications_agree_bit_for_bit(lib, chamber, n_sub, leaf, m):
         assert torch.equal(P.oras_apply(X).cpu(), ref)
     for c in range(0, m, 32):
         assert torch.equal(P.oras_apply(X[:, c:c + 32].contiguous()).cpu(), ref[:, c:c + 32])
+    P.close()
+
+
+def test_an_expired_wait_is_reported_and_the_problem_stays_usable(lib, chamber):
+    """No looks at the dependencies' counts: every tile that depends on another
+    one gives up at once, the launch returns, the host reads the status, and the
+    next call with the default limit gives the earlier result bit for bit."""
+    M, eps = chamber
+    P = lib.Problem(M, eps, FREQ, n_sub=7, precision=1, rtol=1e-9, max_iter=60)
+    ants = antenna_array(ring_antennas(5, radius=0.1))
+    X = _block(M.ndof, 40, 6)
+    ref, S = P.oras_apply(X).cpu(), P.forward_solve(ants, ants)
+    for _ in range(2):
+        P.set_sweep_polls(0)
+        for call in (lambda: P.oras_apply(X), lambda: P.forward_solve(ants, ants)):
+            with pytest.raises(lib.MwiError) as err:
+                call()
+            assert err.value.status == lib.MWI_ETIMEOUT
+        P.set_sweep_polls(-1)
+        assert torch.equal(P.oras_apply(X).cpu(), ref)
+        assert np.array_equal(P.forward_solve(ants, ants), S)
     P.close()
