@@ -1413,6 +1413,7 @@ mwi_status mwi_forward_solve(mwi_problem_t P, const mwi_antenna* tx, int32_t n_t
         }
         P->Brhs.ensure(nm);
         P->U.ensure(nm);
+        P->have_fwd = P->have_adj = false;  // until U and S are this call's
         MWI_CUDA(cudaMemsetAsync(P->Brhs.p, 0, nm * sizeof(double2), st));
         launch_rhs(m, P->tx_dof_d.p, P->tx_sign_d.p, P->cur_d.p, 2.0 * kPi * P->freq * kMu0, P->Brhs.p, st);
         P->m_fwd = m;
@@ -1421,13 +1422,13 @@ mwi_status mwi_forward_solve(mwi_problem_t P, const mwi_antenna* tx, int32_t n_t
         P->rec_m[0] = 0;
         try {
             solve_columns(P, P->Brhs.p, P->U.p, m, info, rec);
-            P->rec_m[0] = m;
         } catch (const Error& e) {
             if (e.status != MWI_ENOTCONV) throw;
             status = MWI_ENOTCONV;
             set_last_error(e.what());
         }
         check_sweep_error(P);
+        if (status == MWI_OK) P->rec_m[0] = m;
         P->S_d.ensure((size_t)n_rx * m);
         launch_s_extract(n_rx, m, P->rx_dof_d.p, P->rx_sign_d.p, P->U.p, P->S_d.p, st);
         MWI_CUDA(cudaMemcpyAsync(S_out, P->S_d.p, (size_t)n_rx * m * sizeof(double2), cudaMemcpyDeviceToHost, st));
@@ -1474,13 +1475,13 @@ static void misfit_and_adjoint(mwi_problem_t P, const double* S_meas, const doub
     P->rec_m[1] = 0;
     try {
         solve_columns(P, P->Brhs.p, P->Lam.p, m, info, rec, fwd);
-        P->rec_m[1] = m;
     } catch (const Error& e) {
         if (e.status != MWI_ENOTCONV) throw;
         status = MWI_ENOTCONV;
         set_last_error(e.what());
     }
     check_sweep_error(P);
+    if (status == MWI_OK) P->rec_m[1] = m;
 }
 
 static mwi_status misfit_grad_impl(mwi_problem_t P, const double* S_meas, const double* w, double* J_out,

@@ -69,3 +69,25 @@ def test_an_expired_wait_is_reported_and_the_problem_stays_usable(lib, chamber):
         assert torch.equal(P.oras_apply(X).cpu(), ref)
         assert np.array_equal(P.forward_solve(ants, ants), S)
     P.close()
+
+
+def test_a_failed_solve_leaves_no_fields_behind(lib, chamber):
+    """A forward solve that gives up has overwritten the fields of the one
+    before: asking for a gradient of them is a call out of order, and the next
+    solve is not recycled from them."""
+    M, eps = chamber
+    P = lib.Problem(M, eps, FREQ, n_sub=7, precision=1, rtol=1e-9, max_iter=60, recycle=1)
+    ants = antenna_array(ring_antennas(5, radius=0.1))
+    S = P.forward_solve(ants, ants)
+    P.misfit_and_gradient(S * 1.1)
+    P.set_sweep_polls(0)
+    with pytest.raises(lib.MwiError) as err:
+        P.forward_solve(ants, ants)
+    assert err.value.status == lib.MWI_ETIMEOUT
+    P.set_sweep_polls(-1)
+    for call in (lambda: P.misfit_and_gradient(S * 1.1), lambda: P.fields(0), lambda: P.fields(1)):
+        with pytest.raises(lib.MwiError) as err:
+            call()
+        assert err.value.status == lib.MWI_ESTATE
+    assert np.array_equal(P.forward_solve(ants, ants), S)
+    P.close()
