@@ -111,7 +111,7 @@ constexpr int kSmemBytes =
     kStages * kStage + 1024 /* barriers */ + kRing * 128 + kSurBufs * kUrCache * 4 + 1024 /* alignment */;
 static_assert((3 * kStages + 4 + 2 * kRing + kSurBufs + 1) * 8 + 8 <= 1024, "barriers");
 static_assert(kSmemBytes * kCtasPerSm <= 228 * 1024 - 2048, "shared memory per SM");
-constexpr long long kWaitLimit = 1ll << 24;
+constexpr int kWaitLimit = 1 << 24;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -138,7 +138,7 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
 // bounded wait on a phase; false if the CTA aborts or the limit expires
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err,
                                           int code) {
-    for (long long it = 0; it < kWaitLimit; ++it) {
+    for (int it = 0; it < kWaitLimit; ++it) {
         if (mbar_try(bar, parity)) return true;  // try_wait suspends in hardware for a while
         if (*abort_flag) return false;
         if (it > (1 << 20)) __nanosleep(256);
@@ -237,11 +237,19 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 __device__ __forceinline__ void red_release(int* p) {
     asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p) : "memory");
 }
-// the same answer in every lane, so that a warp whose lanes see the abort at
-// different times leaves its loop as one (its warp-wide instructions need them all)
+// The same for a whole warp, which has to leave its loop as one, since its
+// warp-wide instructions need all lanes, while lanes may see the abort at
+// different times: they look together and take the decision by votes.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err,
                                                int code) {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, err, code));
+    for (int it = 0; it < kWaitLimit; ++it) {
+        if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+        if (__any_sync(0xffffffffu, *abort_flag)) return false;
+        if (it > (1 << 20)) __nanosleep(256);
+    }
+    *abort_flag = 1;
+    atomicExch(err, code);
+    return false;
 }
 // bounded wait without the abort: for what is in flight when the CTA ends
 __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
@@ -400,12 +408,16 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
     const uint32_t tmem = *tmem_slot;
     const int total = ntiles * nchunks;
 
+    // what a role has under way, for the end of a CTA that gives up: stages copied or
+    // multiplied, tiles multiplied, index buffers filled
+    long long g = 0;
+    int done = 0, nsur = 0;
+    bool ok = true;
+
     if (warp == 0) {
         // ---------------- panel blocks
-        long long g = 0;
-        bool ok = true;
         for (int it = 0; ok; ++it) {
-            if (!(ok = mbar_wait_warp(tile_bar(it), tile_par(it), abort_flag, err, 8))) break;
+            if (!mbar_wait_warp(tile_bar(it), tile_par(it), abort_flag, err, 8)) break;
             const RingSlot* slot = ring + (it & (kRing - 1));
             if (!slot->valid) break;
             const TcGeom G = tc_geom(slot->d.p, slot->d.f, slot->d.row0, slot->d.bwd != 0);
@@ -415,26 +427,19 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                 const int s = (int)(g % kStages);
                 const uint32_t ph = (uint32_t)((g / kStages) & 1);
                 if (!(ok = mbar_wait_warp(empty_bar(s), ph ^ 1, abort_flag, err, 1))) break;
+                // the barrier's one arrival keeps the phase open, whichever comes first, the
+                // count of the expected bytes or another lane's copy
                 const int k0 = G.k0 + st * kKS, nk = min(kKS, G.k0 + G.nk - k0);
                 if (lane == 0) mbar_arrive_tx(raw_bar(s), a_bytes * nk);
-                __syncwarp();
                 if (lane < nk)
                     bulk_g2s(sbase + s * kStage + lane * 8192, P + ((int64_t)(k0 + lane) * G.cstride + G.g0) * 128,
                              a_bytes, raw_bar(s));
                 if (st == 0 && lane == 0) mbar_arrive(begun_bar);
             }
         }
-        // copies still in flight land before the CTA gives its shared memory back, also
-        // when this warp is through and another one has given up
-        if (lane == 0)
-            for (long long q = g > kStages ? g - kStages : 0; q < g; ++q)
-                mbar_drain(raw_bar((int)(q % kStages)), (uint32_t)((q / kStages) & 1));
     } else if (warp == 1) {
         // ---------------- tensor-core products
         if (lane == 0) {
-            long long g = 0;
-            int done = 0;  // tiles multiplied
-            bool ok = true;
             constexpr uint32_t kIdesc = idesc_tf32(128, 64);
             for (int it = 0; ok; ++it) {
                 if (!mbar_wait(tile_bar(it), tile_par(it), abort_flag, err, 8)) break;
@@ -467,19 +472,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                 mma_commit(tfull_bar(buf));
                 ++done;
             }
-            // products and commits still in flight, before the tensor memory is freed
-            for (long long q = g > kStages ? g - kStages : 0; q < g; ++q)
-                mbar_drain(empty_bar((int)(q % kStages)), (uint32_t)((q / kStages) & 1));
-            for (int q = max(0, done - 2); q < done; ++q) mbar_drain(tfull_bar(q & 1), (uint32_t)(q >> 1) & 1);
         }
     } else if (warp < 4) {
         // ---------------- right-hand-side rows into the B operand: this warp's half
         // of the stage's K rows
         constexpr int kMine = kKRows / 4;  // row pairs of a stage per warp
         const int seg = lane & 15, half = lane >> 4, first = (warp - 2) * (kKRows / 2) + half;
-        long long g = 0;
-        int nsur = 0;
-        bool ok = true;
         for (int it = 0; ok; ++it) {
             if (!mbar_wait_warp(tile_bar(it), tile_par(it), abort_flag, err, 8)) break;
             const RingSlot* slot = ring + (it & (kRing - 1));
@@ -493,9 +491,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             const int32_t* iu = urows + slot->d.u_off;
             const int kfirst = G.bwd ? G.row0 : 0;
             if (indices_cached(G)) {
-                if (!(ok = mbar_wait_warp(sur_bar(nsur % kSurBufs), (uint32_t)(nsur / kSurBufs) & 1, abort_flag, err,
-                                          6)))
-                    break;
+                if (!mbar_wait_warp(sur_bar(nsur % kSurBufs), (uint32_t)(nsur / kSurBufs) & 1, abort_flag, err, 6)) break;
                 iu = sur + (nsur % kSurBufs) * kUrCache + (slot->d.u_off & 3);
                 ++nsur;
             }
@@ -503,7 +499,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             // as well, learns from warp 2 that they are there
             const int dep = lane == 0 ? slot->d.dep0 : (lane == 1 ? slot->d.dep1 : -1);
             const int need = lane == 0 ? slot->d.need0 : slot->d.need1;
-            if (!(ok = dep_wait_warp(dep >= 0 ? cnt + dep : nullptr, need * nchunks, polls, abort_flag, err, 7))) break;
+            if (!dep_wait_warp(dep >= 0 ? cnt + dep : nullptr, need * nchunks, polls, abort_flag, err, 7)) break;
             if (warp == 2 && lane == 0) mbar_arrive(deps_bar(it));
             for (int st = 0; st < G.nst; ++st, ++g) {
                 const int s = (int)(g % kStages);
@@ -541,7 +537,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
         // i - 1 are under way, i.e. after the products of the stage kStages before,
         // which is of tile i - 1 - kStages or later: that tile's rows are gathered,
         // and its accumulator waited for the epilogue of the tile two before.
-        int nsur = 0;  // index buffers filled so far
         for (int it = 0;; ++it) {
             if (it > 0 && !mbar_wait_warp(begun_bar, (uint32_t)(it - 1) & 1, abort_flag, err, 10)) break;
             const int tk = __shfl_sync(0xffffffffu, lane == 0 ? atomicAdd(cnt, 1) : 0, 0);
@@ -566,15 +561,11 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             }
             nsur += indices_cached(G) ? 1 : 0;
         }
-        if (lane == 0)
-            for (int q = max(0, nsur - kSurBufs); q < nsur; ++q)
-                mbar_drain(sur_bar(q % kSurBufs), (uint32_t)(q / kSurBufs) & 1);
     } else {
         // ---------------- epilogue
         const int lg = warp & 3;  // tensor-memory lane group of this warp
         const int i = lg * 32 + lane;
-        bool ok = true;
-        for (int it = 0; ok; ++it) {
+        for (int it = 0;; ++it) {
             if (!mbar_wait_warp(tile_bar(it), tile_par(it), abort_flag, err, 8)) break;
             const RingSlot* slot = ring + (it & (kRing - 1));
             if (!slot->valid) break;
@@ -599,14 +590,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             }
             if (d.sib >= 0 && __any_sync(0xffffffffu, add)) {
                 // the second child adds to the parent's rows after the first
-                if (!(ok = dep_wait_warp(lane == 0 ? cnt + d.sib : nullptr, d.needs * nchunks, polls, abort_flag, err,
-                                         9)))
+                if (!dep_wait_warp(lane == 0 ? cnt + d.sib : nullptr, d.needs * nchunks, polls, abort_flag, err,
+                                   9))
                     break;
             }
-            if (!(ok = mbar_wait_warp(tfull_bar(buf), (it >> 1) & 1, abort_flag, err, 5))) break;
-            // past already (the product came after it): orders this lane's reads of the
-            // children's rows after the gather warp's acquire
-            if (!(ok = mbar_wait_warp(deps_bar(it), tile_par(it), abort_flag, err, 11))) break;
+            // the second is past already (the product came after it): it orders this lane's
+            // reads of the children's rows after the gather warp's acquire
+            if (!mbar_wait_warp(tfull_bar(buf), (it >> 1) & 1, abort_flag, err, 5)) break;
+            if (!mbar_wait_warp(deps_bar(it), tile_par(it), abort_flag, err, 11)) break;
             tc_fence_after();
             const uint32_t t0 = tmem + ((uint32_t)(lg * 32) << 16) + buf * 128;
             // whole 32-byte accesses: a lane's row is a line of its own, so an access
@@ -689,6 +680,23 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
     }
     tc_fence_before();
     __syncthreads();
+    if (*abort_flag) {
+        // copies still on their way land before the CTA gives its shared memory back,
+        // products before it frees the tensor memory (every role has stopped; the flag
+        // is the same for all threads)
+        if (lane == 0) {
+            for (long long q = g > kStages ? g - kStages : 0; q < g; ++q) {
+                const uint32_t ph = (uint32_t)((q / kStages) & 1);
+                if (warp == 0) mbar_drain(raw_bar((int)(q % kStages)), ph);
+                if (warp == 1) mbar_drain(empty_bar((int)(q % kStages)), ph);
+            }
+            for (int q = max(0, done - 2); q < done; ++q) mbar_drain(tfull_bar(q & 1), (uint32_t)(q >> 1) & 1);
+            if (warp == 8)
+                for (int q = max(0, nsur - kSurBufs); q < nsur; ++q)
+                    mbar_drain(sur_bar(q % kSurBufs), (uint32_t)(q / kSurBufs) & 1);
+        }
+        __syncthreads();
+    }
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
