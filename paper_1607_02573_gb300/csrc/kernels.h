@@ -198,6 +198,7 @@ int64_t tiled_panel_floats(int p, int f);
 // both tiled copies: the forward one at wt, the backward one at wt + bwd_base
 void pack_tiled(const int2* blocks, int64_t nblocks, const int64_t* f_off, const int64_t* t_off, const int32_t* P,
                 const int32_t* U, const float2* ws, float* wt, int64_t bwd_base, cudaStream_t st);
+// rows of Y come back biased (tf32.h)
 void sweep_tc_solve(const FrontsDev& F, int m, const float* wt, const float2* dinv, float2* Y, float2* Z,
                     float2* upd, int* cnt, int polls, int* err, cudaStream_t st);
 

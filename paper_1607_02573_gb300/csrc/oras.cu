@@ -17,6 +17,7 @@
 #include "common.h"
 #include "gmres.h"
 #include "kernels.h"
+#include "tf32.h"
 
 namespace mwi {
 
@@ -40,10 +41,11 @@ __global__ void gather_kernel(int64_t nloc, int m, int ld, const int32_t* __rest
     Y[e] = c < m ? cvt<In, C>(x[(int64_t)loc2glob[r] * m + c]) : czero<C>();
 }
 
+// biased: Y comes from the tensor-core sweeps (tf32.h)
 template <typename C, typename Out>
 __global__ void scatter_kernel(int64_t n, int m, int ld, const int64_t* __restrict__ own_ptr,
                                const int32_t* __restrict__ own_row, const double* __restrict__ own_w,
-                               const C* __restrict__ Y, Out* __restrict__ y) {
+                               const C* __restrict__ Y, Out* __restrict__ y, int biased) {
     int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= n * m) return;
     int64_t g = e / m;
@@ -52,6 +54,8 @@ __global__ void scatter_kernel(int64_t n, int m, int ld, const int64_t* __restri
     C acc = czero<C>();
     for (int64_t q = own_ptr[g]; q < own_ptr[g + 1]; ++q) {
         C v = Y[(int64_t)own_row[q] * ld + c];
+        if constexpr (std::is_same<C, float2>::value)
+            if (biased) v = make_float2(tf32_unbias(v.x), tf32_unbias(v.y));
         R w = (R)own_w[q];
         acc.x += w * v.x;
         acc.y += w * v.y;
@@ -77,14 +81,15 @@ __global__ void gather2_kernel(int64_t nloc, int h, int ldh, const int32_t* __re
 
 __global__ void scatter2_kernel(int64_t n, int h, int ldh, const int64_t* __restrict__ own_ptr,
                                 const int32_t* __restrict__ own_row, const double* __restrict__ own_w,
-                                const float4* __restrict__ Y, float4* __restrict__ y) {
+                                const float4* __restrict__ Y, float4* __restrict__ y, int biased) {
     const int64_t g = blockIdx.x * (int64_t)blockDim.y + threadIdx.y;
     if (g >= n) return;
     const int64_t q0 = own_ptr[g], q1 = own_ptr[g + 1];
     for (int c = threadIdx.x; c < h; c += blockDim.x) {
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int64_t q = q0; q < q1; ++q) {
-            const float4 v = Y[(int64_t)own_row[q] * ldh + c];
+            float4 v = Y[(int64_t)own_row[q] * ldh + c];
+            if (biased) v = make_float4(tf32_unbias(v.x), tf32_unbias(v.y), tf32_unbias(v.z), tf32_unbias(v.w));
             const float w = (float)own_w[q];
             acc.x += w * v.x;
             acc.y += w * v.y;
@@ -115,7 +120,8 @@ static void oras_apply_impl(const FrontsDev& F, const C* ws, const In* x, Out* y
                          std::is_same<Out, float2>::value;
     const bool pairs = c64 && (m % 2) == 0 && (ld % 2) == 0;
     const int64_t n = (int64_t)F.own_ptr.n - 1;
-    int* cnt = std::is_same<C, float2>::value && sc.tc == 4 ? sc.cnt : nullptr;
+    const int tc4 = std::is_same<C, float2>::value && sc.tc == 4 ? 1 : 0;
+    int* cnt = tc4 ? sc.cnt : nullptr;
     const int ncnt = (int)F.tc_counts();
     if (pairs) {
         const dim3 b = pair_block(m / 2);
@@ -134,11 +140,11 @@ static void oras_apply_impl(const FrontsDev& F, const C* ws, const In* x, Out* y
         const dim3 b = pair_block(m / 2);
         scatter2_kernel<<<(unsigned)((n + b.y - 1) / b.y), b, 0, st>>>(
             n, m / 2, ld / 2, F.own_ptr.p, F.own_row.p, F.own_w.p, reinterpret_cast<const float4*>(Y),
-            reinterpret_cast<float4*>(y));
+            reinterpret_cast<float4*>(y), tc4);
     } else {
         const int64_t tot = n * m;
         scatter_kernel<C, Out><<<(unsigned)((tot + th - 1) / th), th, 0, st>>>(n, m, ld, F.own_ptr.p, F.own_row.p,
-                                                                              F.own_w.p, Y, y);
+                                                                              F.own_w.p, Y, y, tc4);
     }
     MWI_CHECK_LAUNCH();
 }

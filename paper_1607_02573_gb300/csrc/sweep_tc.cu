@@ -31,8 +31,15 @@
 // and the right-hand sides B stored as reals [k][2c + (0 re, 1 im)], the MMA
 // computes Dr = Ar B and Di = Ai B (N = 64 real columns for 32 complex
 // columns, TF32 inputs -- the tensor core reads the FP32 bits and drops the
-// low 13 mantissa bits -- FP32 accumulation); then
+// low 13 mantissa bits, see Rounding below -- FP32 accumulation); then
 //   Re C(i, c) = Dr[i][2c] - Di[i][2c+1],  Im C(i, c) = Dr[i][2c+1] + Di[i][2c].
+//
+// Rounding.  The panels are rounded to the nearest TF32 value when they are
+// packed.  The rows that the backward sweep reads are FP32 words biased by half a
+// TF32 unit (tf32.h), so that the truncation rounds them to nearest as well: Z,
+// which nothing else reads, and the pivot rows of Y that the backward tiles
+// write, which come back biased and whose reader takes the bias off again
+// (oras.cu).  The forward sweep's rows are truncated.
 //
 // Kernel: one launch for both sweeps over the whole tree, two CTAs per SM.
 // Every CTA draws tiles (front, 128-row tile, 32-column chunk) from one list by
@@ -88,6 +95,7 @@
 
 #include "common.h"
 #include "kernels.h"
+#include "tf32.h"
 
 namespace mwi {
 namespace {
@@ -148,6 +156,20 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return false;
 }
 
+// The same for a whole warp, which has to leave its loop as one, since its
+// warp-wide instructions need all lanes, while lanes may see the abort at
+// different times: they look together and take the decision by votes.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err,
+                                               int code) {
+    for (int it = 0; it < kWaitLimit; ++it) {
+        if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+        if (__any_sync(0xffffffffu, *abort_flag)) return false;
+        if (it > (1 << 20)) __nanosleep(256);
+    }
+    *abort_flag = 1;
+    atomicExch(err, code);
+    return false;
+}
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(bar)
@@ -236,20 +258,6 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 }
 __device__ __forceinline__ void red_release(int* p) {
     asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p) : "memory");
-}
-// The same for a whole warp, which has to leave its loop as one, since its
-// warp-wide instructions need all lanes, while lanes may see the abort at
-// different times: they look together and take the decision by votes.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err,
-                                               int code) {
-    for (int it = 0; it < kWaitLimit; ++it) {
-        if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
-        if (__any_sync(0xffffffffu, *abort_flag)) return false;
-        if (it > (1 << 20)) __nanosleep(256);
-    }
-    *abort_flag = 1;
-    atomicExch(err, code);
-    return false;
 }
 // bounded wait without the abort: for what is in flight when the CTA ends
 __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
@@ -491,7 +499,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             const int32_t* iu = urows + slot->d.u_off;
             const int kfirst = G.bwd ? G.row0 : 0;
             if (indices_cached(G)) {
-                if (!mbar_wait_warp(sur_bar(nsur % kSurBufs), (uint32_t)(nsur / kSurBufs) & 1, abort_flag, err, 6)) break;
+                if (!mbar_wait_warp(sur_bar(nsur % kSurBufs), (uint32_t)(nsur / kSurBufs) & 1, abort_flag, err, 6))
+                    break;
                 iu = sur + (nsur % kSurBufs) * kUrCache + (slot->d.u_off & 3);
                 ++nsur;
             }
@@ -604,12 +613,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             // of the warp takes 32 passes whatever its width (32 columns, 402,444 tets:
             // 1.82 -> 1.75 ms; 64 columns 2.93 -> 2.72 ms)
             const bool wide = nc == 32 && (m & 3) == 0;
-            // two halves of 16 complex columns: tensor-memory loads, combine,
-            // D^{-1} or the rows to add, stores; the accumulator is released
-            // once the second half is in registers.  Rows that other tiles of
-            // this launch have written are read past L1.
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            // one or two halves of 16 complex columns: tensor-memory loads, combine,
+            // D^{-1} or the rows to add, stores; the accumulator is released once
+            // the last half is in registers.  Rows that other tiles of this launch
+            // have written are read past L1.  Not unrolled: two copies of the body
+            // are more than the instruction cache takes beside the other roles
+            // (32 columns, 402,444 tets: 1.65 -> 1.55 ms per application).
+#pragma unroll 1
+            for (int h = 0; 16 * h < nc; ++h) {
                 __syncwarp();  // lanes without a row left the first half early
                 float o[32];
                 {
@@ -623,13 +634,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                         o[2 * q + 1] = dr[2 * q + 1] + di[2 * q];
                     }
                 }
-                if (h == 1) {
+                if (16 * (h + 1) >= nc) {
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tempty_bar(buf));
                 }
                 const int cb = 16 * h;  // first complex column of the half
-                if (!dst || cb >= nc) continue;
+                if (!dst) continue;
                 if (gi < d.p && !bwd) {
 #pragma unroll
                     for (int q = 0; q < 16; ++q) {
@@ -662,6 +673,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                             o[4 * q + 2] += v.z;
                             o[4 * q + 3] += v.w;
                         }
+                }
+                if (gi < d.p) {  // operands of the backward sweep, Z or Y
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) o[q] = tf32_bias(o[q]);
                 }
                 if (wide) {
 #pragma unroll
@@ -727,7 +742,8 @@ __global__ void __launch_bounds__(256) pack_tiled_kernel(const int2* __restrict_
     const int rg = row >> 3, rl = row & 7;
     for (int kc = 0; kc < P8; ++kc) {
         const int k = kc * 8 + e;
-        const float2 v = (k < p && row < f) ? L[(int64_t)k * f + row] : make_float2(0.f, 0.f);
+        float2 v = (k < p && row < f) ? L[(int64_t)k * f + row] : make_float2(0.f, 0.f);
+        v = make_float2(tf32_round(v.x), tf32_round(v.y));
         float* bf = Tf + ((int64_t)kc * F8 + rg) * 128;   // forward: line = row, element = pivot
         bf[swz32(rl, e)] = v.x;
         bf[64 + swz32(rl, e)] = v.y;
@@ -762,7 +778,7 @@ int sweep_tc_ctas() {
     return n;
 }
 
-// both sweeps; cnt holds F.tc_counts() zeros
+// both sweeps; cnt holds F.tc_counts() zeros; the rows of Y come back biased (tf32.h)
 void sweep_tc_solve(const FrontsDev& F, int m, const float* wt, const float2* dinv, float2* Y, float2* Z,
                     float2* upd, int* cnt, int polls, int* err, cudaStream_t st) {
     static std::once_flag attr;

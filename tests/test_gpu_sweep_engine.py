@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 from synthetic import antenna_array, ring_antennas
-from tests._helpers import FREQ, chamber_case
+from tests._helpers import FREQ, chamber_case, cube_case, rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -91,3 +91,29 @@ def test_a_failed_solve_leaves_no_fields_behind(lib, chamber):
         assert err.value.status == lib.MWI_ESTATE
     assert np.array_equal(P.forward_solve(ants, ants), S)
     P.close()
+
+
+@pytest.mark.parametrize("leaf", [10 ** 6, 16])
+def test_operands_are_rounded_to_nearest(lib, leaf):
+    """Where the forward sweep's operands are TF32 values already, the engine
+    rounds what engine 2 (mma.sync) rounds, both to nearest, so their errors
+    against FP64 are the same up to FP32 summation: right-hand sides of 8-bit
+    integers on the root front alone -- one front over all rows, and a tree of
+    small fronts, whose backward products then read the ancestors' rows.  An
+    operand truncated instead has four times the mean square error (a factor
+    of sqrt((1 + 4) / 2) = 1.58 with one of a product's two): the bound of 1.25
+    lies between."""
+    mesh, eps, _, _ = cube_case(6)
+    M = lib.Mesh(mesh.xyz, mesh.tet, mesh.bface_tag)
+    info = lib.fronts_host(mesh, 1, nd_leaf=leaf)["info"]
+    l2g = lib.decomposition_host(mesh, 1, nd_leaf=leaf)["loc2glob"]
+    root = [r for _, start, p, _, parent in info if parent < 0 for r in range(start, start + p)]
+    rng = np.random.default_rng(8)
+    X = np.zeros((M.ndof, 64), dtype=np.complex128)
+    X[l2g[root]] = (rng.integers(-127, 128, (len(root), 64)) + 1j * rng.integers(-127, 128, (len(root), 64)))
+    out = {}
+    for engine, precision in ((0, 0), (2, 1), (4, 1)):
+        P = lib.Problem(M, eps, FREQ, n_sub=1, precision=precision, sweep_engine=engine, nd_leaf=leaf)
+        out[engine] = P.oras_apply(torch.from_numpy(X).cuda()).cpu().numpy()
+        P.close()
+    assert 0 < rel_err(out[4], out[0]) <= 1.25 * rel_err(out[2], out[0])
