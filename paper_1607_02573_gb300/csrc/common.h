@@ -72,6 +72,12 @@ extern std::atomic<int64_t> g_device_allocs;
         if (!(cond)) throw ::mwi::Error((status), (msg));  \
     } while (0)
 
+inline int current_device() {
+    int dev = 0;
+    MWI_CUDA(cudaGetDevice(&dev));
+    return dev;
+}
+
 // Owning device allocation (cudaMalloc / cudaFree).
 template <typename T>
 struct DevBuf {

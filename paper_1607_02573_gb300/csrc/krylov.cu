@@ -9,13 +9,13 @@
 // all basis vectors with w in one pass, then one fused update pass.
 #include <algorithm>
 #include <cstring>
-#include <mutex>
 #include <type_traits>
 
 #include "common.h"
 #include "df.h"
 #include "gmres.h"
 #include "kernels.h"
+#include "per_device.h"
 
 namespace mwi {
 
@@ -1133,9 +1133,10 @@ void GmresDF::norms2(const float2* xh, double* out, cudaStream_t st) {
 }
 
 static void allow_update_smem() {
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static PerDevice<bool> set;
+    set.get(current_device(), [] {
         MWI_CUDA(cudaFuncSetAttribute(dcgs_update_df2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUpdSmem));
+        return true;
     });
 }
 

@@ -11,12 +11,12 @@
 // Several right-hand sides go through one forward/backward sweep, as the
 // paper notes for multiple vectors (Section 3).  Vectors are row-major [rows][m].
 #include <algorithm>
-#include <mutex>
 #include <type_traits>
 
 #include "common.h"
 #include "gmres.h"
 #include "kernels.h"
+#include "per_device.h"
 #include "tf32.h"
 
 namespace mwi {
@@ -176,21 +176,15 @@ template void oras_apply<double2>(const FrontsDev&, const double2*, const double
 static __device__ __align__(256) unsigned char g_oras_scratch[kOrasScratchBytes];
 
 static void* oras_scratch_address() {
-    int dev = 0;
-    MWI_CUDA(cudaGetDevice(&dev));
-    static std::mutex mu;
-    static std::vector<void*> addr;
-    std::lock_guard<std::mutex> lk(mu);
-    if ((int)addr.size() <= dev) addr.resize(dev + 1, nullptr);
-    if (!addr[dev]) {
+    static PerDevice<void*> addr;
+    return addr.get(current_device(), [] {
         void* p = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&p, g_oras_scratch);
         if (e != cudaSuccess || !p)
             throw Error(MWI_ECUDA, std::string("cudaGetSymbolAddress of the ORAS scratch failed: ") +
                                        cudaGetErrorString(e));
-        addr[dev] = p;
-    }
-    return addr[dev];
+        return p;
+    });
 }
 
 static size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }

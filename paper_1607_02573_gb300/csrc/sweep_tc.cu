@@ -91,10 +91,10 @@
 // the CTA lets its copies and products in flight land, frees its tensor memory
 // and returns.
 #include <algorithm>
-#include <mutex>
 
 #include "common.h"
 #include "kernels.h"
+#include "per_device.h"
 #include "tf32.h"
 
 namespace mwi {
@@ -767,29 +767,27 @@ void pack_tiled(const int2* blocks, int64_t nblocks, const int64_t* f_off, const
     }
 }
 
-int sweep_tc_ctas() {
-    static int n = 0;
-    if (!n) {
-        int dev = 0, sms = 0;
-        MWI_CUDA(cudaGetDevice(&dev));
+// CTAs of a launch on the current device, and the kernel's shared memory allowed there
+static int sweep_tc_ctas() {
+    static PerDevice<int> ctas;
+    const int dev = current_device();
+    return ctas.get(dev, [dev] {
+        int sms = 0;
         MWI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        n = std::max(1, sms * kCtasPerSm);
-    }
-    return n;
+        MWI_CUDA(cudaFuncSetAttribute(sweep_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+        return std::max(1, sms * kCtasPerSm);
+    });
 }
 
 // both sweeps; cnt holds F.tc_counts() zeros; the rows of Y come back biased (tf32.h)
 void sweep_tc_solve(const FrontsDev& F, int m, const float* wt, const float2* dinv, float2* Y, float2* Z,
                     float2* upd, int* cnt, int polls, int* err, cudaStream_t st) {
-    static std::once_flag attr;
-    std::call_once(attr, [] {
-        MWI_CUDA(cudaFuncSetAttribute(sweep_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-    });
+    const int ctas = sweep_tc_ctas();
     const int nchunks = (m + 31) / 32;
     const int64_t total = F.tc_ntiles * nchunks;
-    MWI_REQUIRE(total + 2 * sweep_tc_ctas() < ((int64_t)1 << 31), MWI_EINVAL, "too many sweep tiles");
+    MWI_REQUIRE(total + 2 * ctas < ((int64_t)1 << 31), MWI_EINVAL, "too many sweep tiles");
     if (total <= 0) return;
-    const int grid = (int)std::min<int64_t>(total, sweep_tc_ctas());
+    const int grid = (int)std::min<int64_t>(total, ctas);
     sweep_tc_kernel<<<grid, kThreads, kSmemBytes, st>>>(F.tc_tiles.p, (int)F.tc_ntiles, nchunks, cnt, F.urows.p,
                                                         F.asm2.p, F.pdst.p, wt, dinv, Y, Z, upd, m, polls, err);
     MWI_CHECK_LAUNCH();
