@@ -371,7 +371,7 @@ def run_mine(args, rank, world):
 # from ncu's dram__bytes_read.sum + dram__bytes_write.sum (tcgen05 sweeps,
 # nested-dissection leaf 128)
 ORAS_TRAFFIC = {"bytes_per_call": 8.064e9,
-                "source": "ncu DRAM counters of one apply at the bench size, profiles/oras_apply_chamber402k_traffic.md"}
+                "source": "ncu DRAM counters of one apply at the bench size"}
 
 
 def db_bins(S, S_ref, edges=(0.0, -20.0, -60.0)):

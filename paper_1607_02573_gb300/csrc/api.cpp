@@ -422,16 +422,15 @@ std::shared_ptr<DecompEntry> get_decomp(mwi_mesh* M, const mwi_solver_opts& o) {
 void upload_fronts(const Decomposition& D, FrontsDev& F, cudaStream_t st) {
     const size_t nf = D.fronts.size();
     F.nfronts = (int64_t)nf;
-    std::vector<int32_t> start(nf), p(nf), u(nf), parent(nf), sub(nf);
-    std::vector<int64_t> f_off(nf), u_off(nf), upd_row(nf), sch_off(nf);
+    std::vector<int32_t> start(nf), p(nf), u(nf), sub(nf);
+    std::vector<int64_t> f_off(nf), u_off(nf), sch_off(nf);
     for (size_t k = 0; k < nf; ++k) {
         const Front& fr = D.fronts[k];
-        start[k] = fr.start; p[k] = fr.p; u[k] = fr.u; parent[k] = fr.parent; sub[k] = fr.sub;
-        f_off[k] = fr.f_off; u_off[k] = fr.u_off; upd_row[k] = fr.upd_row; sch_off[k] = fr.sch_off;
+        start[k] = fr.start; p[k] = fr.p; u[k] = fr.u; sub[k] = fr.sub;
+        f_off[k] = fr.f_off; u_off[k] = fr.u_off; sch_off[k] = fr.sch_off;
     }
-    up(F.start, start, st); up(F.p, p, st); up(F.u, u, st); up(F.parent, parent, st); up(F.sub, sub, st);
-    up(F.f_off, f_off, st); up(F.u_off, u_off, st); up(F.upd_row, upd_row, st); up(F.sch_off, sch_off, st);
-    up(F.child_ptr, D.child_ptr, st); up(F.child, D.child, st);
+    up(F.start, start, st); up(F.p, p, st); up(F.u, u, st); up(F.sub, sub, st);
+    up(F.f_off, f_off, st); up(F.u_off, u_off, st); up(F.sch_off, sch_off, st);
     {
         // padded: the sweeps copy index lists in 16-byte units
         std::vector<int32_t> ur(D.urows);
@@ -439,7 +438,6 @@ void upload_fronts(const Decomposition& D, FrontsDev& F, cudaStream_t st) {
         up(F.urows, ur, st);
     }
     up(F.urel, D.urel, st);
-    up(F.asm_base, D.asm_base, st); up(F.asm_ptr, D.asm_ptr, st); up(F.asm_src, D.asm_src, st);
     {
         // every front row receives at most one row from each of its (at most two) children
         const int64_t rows = (int64_t)D.asm_ptr.size() - 1;

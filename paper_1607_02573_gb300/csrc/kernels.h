@@ -111,13 +111,10 @@ struct FrontsDev {
     DevBuf<int64_t> t_off;
     DevBuf<int2> pack_blocks;
     int64_t n_pack_blocks = 0, tiled_floats = 0;
-    DevBuf<int32_t> start, p, u, parent, sub;
-    DevBuf<int64_t> f_off, u_off, upd_row, sch_off;
-    DevBuf<int32_t> child_ptr, child;
+    DevBuf<int32_t> start, p, u, sub;
+    DevBuf<int64_t> f_off, u_off, sch_off;
     DevBuf<int32_t> urows, urel;
-    DevBuf<int64_t> asm_base, asm_ptr;   // gather lists of the sweeps' extend-add
-    DevBuf<int32_t> asm_src;
-    DevBuf<int2> asm2;                   // the same lists as (source, source) per front row, -1 = none
+    DevBuf<int2> asm2;                   // the sweeps' extend-add: (source, source) per front row, -1 = none
     // extend-add tiles (front, child, first of four child rows), per level and
     // chunk of 65535 fronts: first children, then second children
     DevBuf<int4> ext_tiles;

@@ -132,8 +132,7 @@ __global__ void __launch_bounds__(256) dots_kernel(int64_t n, int m, int nvec_in
 }
 
 // h[i][c] = sum_b partial[b][i][c] for i < nvec; hacc[i][c] += h[i][c] for i < nacc;
-// hdf (optional) receives h as double-floats (re hi, re lo, im hi, im lo); clear
-// (optional): two counters set to zero on the way.
+// clear (optional): two counters set to zero on the way.
 // One block per vector index i: 32 warps split the blocks b (b = warp, warp +
 // 32, ...), lanes over columns, then a fixed-order sum of the 32 partial sums.
 // The chain of loads and FP64 additions per warp bounds it (with 8 warps a
@@ -141,7 +140,7 @@ __global__ void __launch_bounds__(256) dots_kernel(int64_t n, int m, int nvec_in
 __global__ void __launch_bounds__(1024) dots_reduce_kernel(int nblk, int nvec, int nacc, int m,
                                                           const double2* __restrict__ partial,
                                                           double2* __restrict__ h, double2* __restrict__ hacc,
-                                                          float4* __restrict__ hdf, int* __restrict__ clear) {
+                                                          int* __restrict__ clear) {
     __shared__ double2 red[32][33];
     const int i = blockIdx.x;
     if (clear && i == 0 && threadIdx.x < 2) clear[threadIdx.x] = 0;
@@ -168,10 +167,6 @@ __global__ void __launch_bounds__(1024) dots_reduce_kernel(int nblk, int nvec, i
             const int e = i * m + c;
             h[e] = s;
             if (hacc && i < nacc) { hacc[e].x += s.x; hacc[e].y += s.y; }
-            if (hdf) {
-                const float2 a = df_split(s.x), b = df_split(s.y);
-                hdf[e] = make_float4(a.x, a.y, b.x, b.y);
-            }
         }
         __syncthreads();
     }
@@ -548,48 +543,6 @@ __global__ void __launch_bounds__(256) spmm_df2_kernel(int64_t n, const int32_t*
         Wh[row * h + c] = make_float4(re0.h, im0.h, re1.h, im1.h);
         Wl[row * h + c] = make_float4(re0.l, im0.l, re1.l, im1.l);
     }
-}
-
-// W -= sum_i V_i h_i per column (V_i and W double-float, h double-float
-// [nvec][m] as (re hi, re lo, im hi, im lo)); four basis vectors per step so
-// that their loads are in flight together
-__global__ void __launch_bounds__(256) cgs_update_df_kernel(int64_t nm, int m, int nvec, const float2* __restrict__ V,
-                                                            int64_t vstride, const float4* __restrict__ hdf,
-                                                            float2* __restrict__ W) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= nm) return;
-    const int c = (int)(e % m);
-    const float2 wh = W[e], wl = W[nm + e];
-    dfl re = {wh.x, wl.x}, im = {wh.y, wl.y};
-    int i = 0;
-    for (; i + 4 <= nvec; i += 4) {
-        float2 vh[4], vl[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            vh[u] = V[(int64_t)(i + u) * vstride + e];
-            vl[u] = V[(int64_t)(i + u) * vstride + nm + e];
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const float4 h = hdf[(i + u) * m + c];
-            df_mac(re, -vh[u].x, -vl[u].x, h.x, h.y);
-            df_mac(re, vh[u].y, vl[u].y, h.z, h.w);
-            df_mac(im, -vh[u].x, -vl[u].x, h.z, h.w);
-            df_mac(im, -vh[u].y, -vl[u].y, h.x, h.y);
-        }
-    }
-    for (; i < nvec; ++i) {
-        const float2 vh = V[(int64_t)i * vstride + e], vl = V[(int64_t)i * vstride + nm + e];
-        const float4 h = hdf[i * m + c];
-        df_mac(re, -vh.x, -vl.x, h.x, h.y);
-        df_mac(re, vh.y, vl.y, h.z, h.w);
-        df_mac(im, -vh.x, -vl.x, h.z, h.w);
-        df_mac(im, -vh.y, -vl.y, h.x, h.y);
-    }
-    re = df_norm(re);
-    im = df_norm(im);
-    W[e] = make_float2(re.h, im.h);
-    W[nm + e] = make_float2(re.l, im.l);
 }
 
 // V = W s per column (W, V double-float, s double-float [m])
@@ -1006,24 +959,24 @@ void Gmres<C>::reserve(int64_t n_, int m_, int restart_) {
 }
 
 // out[i][c] = conj(V_i)^T w for i < nvec (+ conj(w)^T w at nvec when self = 1),
-// acc[i] += out[i] for i < nvec, hdf = out as double-floats (optional)
+// acc[i] += out[i] for i < nvec (optional)
 template <typename C>
 static void dots_launch(int64_t n, int m, const C* Vb, int nvec, int64_t vstride, const C* w, double2* partial,
-                        double2* out, double2* acc, float4* hdf, cudaStream_t st, int self) {
+                        double2* out, double2* acc, cudaStream_t st, int self) {
     int mx = 1;
     while (mx < std::min(m, 32)) mx *= 2;
     dim3 blk(mx, 8), grd(kDotBlocks, (m + mx - 1) / mx);
     dots_kernel<C><<<grd, blk, 0, st>>>(n, m, nvec, Vb, vstride, w, self, partial);
     MWI_CHECK_LAUNCH();
     const int nt = nvec + self;
-    dots_reduce_kernel<<<nt, 1024, 0, st>>>(kDotBlocks, nt, nvec, m, partial, out, acc, hdf, nullptr);
+    dots_reduce_kernel<<<nt, 1024, 0, st>>>(kDotBlocks, nt, nvec, m, partial, out, acc, nullptr);
     MWI_CHECK_LAUNCH();
 }
 
 template <typename C>
 void Gmres<C>::dots(const C* Vb, int nvec, int64_t vstride, const C* w, double2* out, double2* acc,
                     cudaStream_t st, int self) {
-    dots_launch<C>(n, m, Vb, nvec, vstride, w, partial.p, out, acc, nullptr, st, self);
+    dots_launch<C>(n, m, Vb, nvec, vstride, w, partial.p, out, acc, st, self);
 }
 
 template <typename C>
@@ -1127,7 +1080,7 @@ void GmresDF::reserve(int64_t n_, int m_, int restart_) {
 }
 
 void GmresDF::norms2(const float2* xh, double* out, cudaStream_t st) {
-    dots_launch<float2>(n, m, xh, 0, 0, xh, partial.p, h.p, nullptr, nullptr, st, 1);
+    dots_launch<float2>(n, m, xh, 0, 0, xh, partial.p, h.p, nullptr, st, 1);
     real_part_kernel<<<nblocks(m, 128), 128, 0, st>>>(m, h.p, out);
     MWI_CHECK_LAUNCH();
 }
@@ -1176,7 +1129,7 @@ int GmresDF::cycle(const OpA& A, const OpM& M, const float2* r0, float2* x, cons
             dots2_kernel<<<grd, blk, 0, st>>>(n, m, k, V.p, vs, vk, W.p, partial.p);
             MWI_CHECK_LAUNCH();
             const int nout = 2 * k + 3;
-            dots_reduce_kernel<<<nout, 1024, 0, st>>>(nblk, nout, 0, m, partial.p, h.p, nullptr, nullptr, nact);
+            dots_reduce_kernel<<<nout, 1024, 0, st>>>(nblk, nout, 0, m, partial.p, h.p, nullptr, nact);
             MWI_CHECK_LAUNCH();
             arnoldi_dcgs_kernel<<<m, 32, 0, st>>>(m, k, restart, last, h.p, H.p, Hp.p, cs.p, sn.p, g.p, active, kcol,
                                                   tol, resid, rho, nact, hdf.p, hdf2.p, scal.p);
