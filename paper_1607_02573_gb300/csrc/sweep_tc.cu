@@ -616,11 +616,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
             // one or two halves of 16 complex columns: tensor-memory loads, combine,
             // D^{-1} or the rows to add, stores; the accumulator is released once
             // the last half is in registers.  Rows that other tiles of this launch
-            // have written are read past L1.  Not unrolled: two copies of the body
-            // are more than the instruction cache takes beside the other roles
-            // (32 columns, 402,444 tets: 1.65 -> 1.55 ms per application).
-#pragma unroll 1
-            for (int h = 0; 16 * h < nc; ++h) {
+            // have written are read past L1.  The two halves share one copy of the
+            // body: two in a row are more than the instruction cache takes beside the
+            // other roles (32 columns, 402,444 tets: 1.65 ms per application, 1.54
+            // with one).  At most 16 columns get a copy of their own, without the
+            // loop (14 columns, 19k tets: 202 -> 174 us; one column, 7,392 tets:
+            // 125 -> 120 us).
+            auto half = [&](int h) {
                 __syncwarp();  // lanes without a row left the first half early
                 float o[32];
                 {
@@ -640,7 +642,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                     if (lane == 0) mbar_arrive(tempty_bar(buf));
                 }
                 const int cb = 16 * h;  // first complex column of the half
-                if (!dst) continue;
+                if (!dst) return;
                 if (gi < d.p && !bwd) {
 #pragma unroll
                     for (int q = 0; q < 16; ++q) {
@@ -681,13 +683,19 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) sweep_tc_kernel(
                 if (wide) {
 #pragma unroll
                     for (int q = 0; q < 4; ++q) store32(dst + cb + 4 * q, o + 8 * q);
-                    continue;
+                    return;
                 }
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
                     if (cb + 2 * q < nc)
                         reinterpret_cast<float4*>(dst + cb)[q] =
                             make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+                        };
+            if (nc <= 16) {
+                half(0);
+            } else {
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) half(h);
             }
             __syncwarp();
             if (lane == 0) red_release(cnt + d.cnt);
