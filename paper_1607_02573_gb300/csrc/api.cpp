@@ -1465,6 +1465,7 @@ static void misfit_and_adjoint(mwi_problem_t P, const double* S_meas, const doub
     MWI_CUDA(cudaMemsetAsync(P->Brhs.p, 0, nm * sizeof(double2), st));
     launch_adjoint_rhs(n_rx, m, P->rx_dof_d.p, P->rx_sign_d.p, P->r_d.p, wd, P->Brhs.p, st);
     P->Lam.ensure(nm);
+    P->have_adj = false;  // until Lam is this call's
     // recycled space of the adjoint solve: the previous adjoint solutions and
     // the current forward solutions (whose span holds the adjoint solution
     // exactly when the receivers are among the transmitters)

@@ -117,3 +117,23 @@ def test_operands_are_rounded_to_nearest(lib, leaf):
         out[engine] = P.oras_apply(torch.from_numpy(X).cuda()).cpu().numpy()
         P.close()
     assert 0 < rel_err(out[4], out[0]) <= 1.25 * rel_err(out[2], out[0])
+
+
+def test_a_failed_adjoint_solve_leaves_no_adjoint_fields_behind(lib, chamber):
+    M, eps = chamber
+    P = lib.Problem(M, eps, FREQ, n_sub=7, precision=1, rtol=1e-9, max_iter=60)
+    ants = antenna_array(ring_antennas(5, radius=0.1))
+    S_meas = P.forward_solve(ants, ants) * 1.1
+    J, grad = P.misfit_and_gradient(S_meas)
+    P.set_sweep_polls(0)
+    with pytest.raises(lib.MwiError) as err:
+        P.misfit_and_gradient(S_meas)
+    assert err.value.status == lib.MWI_ETIMEOUT
+    P.set_sweep_polls(-1)
+    with pytest.raises(lib.MwiError) as err:
+        P.fields(1)
+    assert err.value.status == lib.MWI_ESTATE
+    P.fields(0)  # the forward fields are still there, and the gradient can be asked for again
+    J2, grad2 = P.misfit_and_gradient(S_meas)
+    assert J2 == J and np.array_equal(grad2, grad)
+    P.close()
