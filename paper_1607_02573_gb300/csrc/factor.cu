@@ -35,9 +35,9 @@
 // is read and written once.  Before, every step updated the whole trailing
 // matrix, and the inverse was formed after the level by column-blocked
 // substitution, eight columns of a front per block, each reading the whole
-// panel.  Whole factorisations, before and now: 3,072 tets 1.34 -> 1.05 ms,
-// 120,288 tets 9.56 -> 8.68 ms, 402,444 tets 39.2 -> 38.0 ms, second order on
-// 53,046 tets 104 -> 82.6 ms, FP64 on 46,080 tets 41.3 -> 38.2 ms.
+// panel.  Whole factorisations (tiled copies included), before and now: 3,072
+// tets 1.34 -> 1.00 ms, 120,288 tets 9.56 -> 8.4 ms, 402,444 tets 39.2 -> 37 ms,
+// second order on 53,046 tets 104 -> 82 ms, FP64 on 46,080 tets 41.3 -> 34.5 ms.
 #include <algorithm>
 #include <type_traits>
 
@@ -239,13 +239,14 @@ __global__ void __launch_bounds__(128, 3) panel_rows_kernel(const int2* __restri
 //   kInv      rows [p, f), columns [0, p): X = -L_i X_1
 // Slabs of KS pivots pass through two shared-memory buffers, the next one's loads
 // in flight during the products.  Complex FP32: bound by the FP32 pipe and by
-// how many warps are there to fill it (half busy at 24 warps per SM): four blocks
-// of 64 registers per SM and slabs of 8 take 38.0 ms per factorisation at 402,444
-// tets, slabs of 16 38.8, three blocks of 80 registers 41.0.  A thread's four rows
-// and columns are the pairs 2t, 2t + 1 and 32 + 2t, 32 + 2t + 1, read as 16-byte
+// how many warps are there to fill it (half to 60 % busy with four blocks of 64
+// registers per SM).  Factorisations of 402,444 tets when the shape was chosen,
+// before the rows kernel worked in place: slabs of 8 and four blocks 38.0 ms,
+// slabs of 16 38.8, three blocks of 80 registers 41.0.  A thread's four rows and
+// columns are the pairs 2t, 2t + 1 and 32 + 2t, 32 + 2t + 1, read as 16-byte
 // shared loads; a complex multiply-add is two packed ones, which halves its issue
-// slots (39.8 -> 39.0 ms; with the packed operands laid out in shared memory,
-// twice the shared loads, 41).
+// slots (at that time 39.8 -> 39.0 ms; with the packed operands laid out in shared
+// memory, twice the shared loads, 41).
 // Complex FP64 is bound by its pipe alone: quarters of a tile without wanted
 // entries -- beyond the last row or column, or above the diagonal -- are left out
 // of the products (46,080 tets: 38.1 -> 34.4 ms per factorisation).  In FP32 the
@@ -438,8 +439,8 @@ void factorize_fronts(const FrontsDev& F, const UpdateTiles& ut, const double2* 
     MWI_REQUIRE(ut.nb == NB && ut.tile == TILE, MWI_EINVAL, "internal: update tiles built for another blocking");
     MWI_CUDA(cudaMemsetAsync(ws, 0, (size_t)(F.ws_entries + F.nloc) * sizeof(C), st));
     const int nlev = (int)F.level_ptr.size() - 1;
-    // the largest front this factorisation accepts, unchanged: 12,800 rows in
-    // complex FP32, 6,400 in FP64
+    // the largest front that is accepted: 12,800 rows in complex FP32, 6,400 in FP64.
+    // Callers have always had this limit; the kernels here do not need it.
     for (int l = 0; l < nlev; ++l)
         MWI_REQUIRE(2 * (size_t)F.level_fmax[l] * sizeof(C) <= 200 * 1024, MWI_EINVAL,
                     "front too large (" + std::to_string(F.level_fmax[l]) + " rows)");

@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(256) spmm_df_kernel(int64_t n, const int32_t* 
 
 // The same product for an even m with two adjacent columns per lane (16-byte
 // loads of the right-hand sides; G lanes per row, the power of two at or above
-// m / 2, at most 16): four independent accumulation chains per thread instead of
+// m / 2, at least 2, at most 16): four independent accumulation chains per thread instead of
 // two.  Entries are applied in the same ascending order, so the results are the
 // same bit for bit.
 // w = A z (RES = false): the error-free products and sums bound it; they run on

@@ -106,8 +106,8 @@ static dim3 pair_block(int h) {
 }
 
 // columns of the local vectors: the tensor-core sweeps move rows by 16-byte
-// bulk copies, so their rows hold an even number of complex FP32 values (an
-// odd m gets one zero column, which every step leaves zero)
+// asynchronous copies, so their rows hold an even number of complex FP32 values (an
+// odd m gets one column of zeros, which no other column sees)
 int sweep_ld(int m, int tc) { return (tc == 4 && (m & 1)) ? m + 1 : m; }
 
 template <typename C, typename In, typename Out>

@@ -608,7 +608,7 @@ void multifrontal_solve(const FrontsDev& F, const C* ws, C* Y, C* Z, C* upd, int
                         cudaStream_t st) {
     if constexpr (std::is_same<C, float2>::value) {
         if (sc.tc == 4) {
-            // the tcgen05 engine moves right-hand-side rows by 16-byte bulk copies
+            // the tcgen05 engine moves right-hand-side rows by 16-byte asynchronous copies
             // (oras_apply pads the local vectors to an even column count)
             MWI_REQUIRE(sc.wt && sc.err && sc.cnt, MWI_EINVAL, "internal: tensor-core sweeps without their buffers");
             MWI_REQUIRE((m % 2) == 0, MWI_EINVAL, "internal: tensor-core sweeps need an even column count");

@@ -63,8 +63,7 @@
 // extend-add of the pivot rows) every level ended in a partly filled last wave
 // and began with the set-up of all CTAs; subdomains, whose levels are
 // independent of each other, now overlap across levels.  Per application of 32
-// columns on 402,444 tets, gather and scatter included: 1.83 -> 1.42 ms; of one
-// column on 7,392 tets 160 -> 70 us.
+// columns on 402,444 tets, gather and scatter included: 1.87 -> 1.38 ms.
 // Warp roles:
 //   warp 0      streams the panel blocks by bulk copies, which depend on no
 //               other tile
